@@ -1,6 +1,7 @@
 // The C ABI of libctrecon (declared in include/ctrecon.h): argument checking,
 // plan construction (fixed-point geometry tables, FFT plan, device workspace),
 // dtype dispatch and stream handling.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -161,6 +162,49 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     // at least two angles per job on average; an odd view count pairs every angle but 0 with
     // its mirror pi - theta ((N + 1) / 2 jobs), which the pair-job kernels serve at half cost
     if (2 * jobs.size() > (size_t)N + 1) return CTR_OK;
+    {
+        size_t pairs = 0;                          // jobs whose angles sit in channels {0, 1} or {2, 3} only
+        for (const OrbitJob &jb : jobs)
+            if ((jb.l[2] < 0 && jb.l[3] < 0) || (jb.l[0] < 0 && jb.l[1] < 0)) ++pairs;
+        p->pair_jobs = 2 * pairs > jobs.size() ? 1 : 0;
+    }
+    // the job lists: one, or the pair jobs of channels {0, 1} and those of {2, 3} (a job with
+    // angles in both becomes two); each sorted by S / C, so that neighbours' rays nearly coincide
+    {
+        std::vector<OrbitJob> lists[2];
+        for (const OrbitJob &jb : jobs) {
+            if (!p->pair_jobs) { lists[0].push_back(jb); continue; }
+            for (int h = 0; h < 2; ++h) {
+                if (jb.l[2 * h] < 0 && jb.l[2 * h + 1] < 0) continue;
+                OrbitJob half = jb;
+                half.l[2 - 2 * h] = half.l[3 - 2 * h] = -1;
+                lists[h].push_back(half);
+            }
+        }
+        jobs.clear();
+        p->job_list[0] = 0;
+        for (int h = 0; h < 2; ++h) {
+            std::stable_sort(lists[h].begin(), lists[h].end(), [](const OrbitJob &x, const OrbitJob &y) {
+                return (__int128)x.am.B * y.am.A < (__int128)y.am.B * x.am.A;
+            });
+            jobs.insert(jobs.end(), lists[h].begin(), lists[h].end());
+            p->job_list[h + 1] = (int)jobs.size();
+        }
+    }
+    const int nc = p->pair_jobs ? 2 : 4;
+    {
+        // orbit-layout rows: every tile's window of obp_win bins, and the detector, inside the row
+        p->obp_win = obp_window(jobs, nc);
+        const long long far = (n + 31) / 32 * 32 - 32;             // origin of the last tile
+        long long lo = 0, hi = M;
+        for (const OrbitJob &jb : jobs) {
+            const long long A = jb.am.A, B = jb.am.B, P = jb.am.Op + ((A + 3 * B) >> 1);
+            lo = std::min(lo, (P >> 32) - 2);
+            hi = std::max(hi, ((P + far * (A + B)) >> 32) - 2 + p->obp_win);
+        }
+        p->bar_pad = ((int)-lo + 4 + 3) & ~3;
+        p->bar_pitch = (p->bar_pad + (int)hi + 3) & ~3;
+    }
     ctr_status st;
     void *tmp = nullptr;
     if ((st = alloc(p, &tmp, sizeof(OrbitJob) * jobs.size())) != CTR_OK) return st;
@@ -179,15 +223,14 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     p->obp_cap = n <= 1024 ? (gmax < MAX_BP_GROUPS ? gmax : MAX_BP_GROUPS) : p->obp_groups;
     if (p->obp_cap < p->obp_groups) p->obp_cap = p->obp_groups;
     if ((st = alloc(p, &p->obp_part, sizeof(float) * 4 * (size_t)p->obp_cap * n * n)) != CTR_OK) return st;
+    const size_t bar_bytes = sizeof(float) * nc * (size_t)p->bar_pitch * jobs.size();
+    for (void **bar : {&p->gbar, &p->ybar}) {
+        if ((st = alloc(p, bar, bar_bytes)) != CTR_OK) return st;
+        CTR_CUDA(cudaMemset(*bar, 0, bar_bytes));                  // the pads stay zero
+    }
     CTR_CUDA(cudaMemcpy(p->d_jobs, jobs.data(), sizeof(OrbitJob) * jobs.size(), cudaMemcpyHostToDevice));
     p->n_jobs = (int)jobs.size();
     p->orbit = true;
-    {
-        size_t pairs = 0;                          // jobs whose angles sit in channels {0, 1} or {2, 3} only
-        for (const OrbitJob &jb : jobs)
-            if ((jb.l[2] < 0 && jb.l[3] < 0) || (jb.l[0] < 0 && jb.l[1] < 0)) ++pairs;
-        p->pair_jobs = 2 * pairs > jobs.size() ? 1 : 0;
-    }
     // the staged forward shape only where its double-buffered window fits one CTA's shared
     // memory (stg_wmax = 0: shape (4, 1) unavailable on this plan)
     p->stg_wmax = stg_window(jobs, n, M);

@@ -280,6 +280,9 @@ struct ForwardEpi {
     T *v1b;            // in/out: bar v1
     T *y1;             // out: bar v1_new + sigma Rt u_new
     __nv_bfloat16 *y1h;   // if set: y1 is stored here in bfloat16 instead (BF16 operand storage)
+    T *ybar;           // if set (symmetric path): y1 is stored here in orbit layout instead ...
+    int ypitch, ypad, ync;   // ... rows of ypitch bins of ync channels, bin 0 at ypad
+    int yround;        // ... rounded through bfloat16 (BF16 plans)
     T *t1;             // optional out: resolvent output (dual certificate)
     const T *dw, *da, *dlo, *dhi;   // per-bin data term, beta-scaled
 };
@@ -311,6 +314,8 @@ struct SliceDesc {
     int n_jobs;
     const OrbitJob *jobs;
     float4 *ubar;
+    const float *ybar;            // the backprojection's operand in orbit layout ...
+    int bar_pitch, bar_pad, obp_win, job_list[3];   // ... its shape and job lists (see ctr_plan)
     BackprojEpi<float> bpe;       // step A epilogue
     ForwardEpi<float> fwe;        // step C epilogue
     float sigma, tau, lam, inv_h;
@@ -399,6 +404,13 @@ struct ctr_plan {
     int obp_groups = 1;                  // job groups of the symmetric backprojection
     int pair_jobs = 0;                   // most jobs are pair jobs: both projectors take their pair variants
     int obp_cap = 1;                     // groups the partial-plane workspace has room for
+    // sinogram operands of the symmetric backprojection in orbit layout: one row per job,
+    // bar_pitch bins of 4 (pair plans: 2) channels, bin 0 at bar_pad, zeros around the detector
+    void *gbar = nullptr;                // operand of a single call
+    void *ybar = nullptr;                // the iteration's y1, written by the forward epilogue
+    int bar_pitch = 0, bar_pad = 0;
+    int obp_win = 0;                     // bins staged per tile and job
+    int job_list[3] = {};                // jobs sorted by S / C: [0, n_jobs), or pair jobs {0, 1} and {2, 3}
     void *obp_part = nullptr;            // obp_groups * 4 * n*n partial planes
     void *d_twiddle = nullptr;  // n complex exp(-2 pi i t/n)
 
@@ -519,7 +531,10 @@ int fwd_grid_y(int N);         // forward-projector grid: angle groups
 
 // batched stages (one launch per stage over all slices of a batch)
 size_t bp_smem_bytes(int wstride);
-size_t obp_smem_bytes(int wstride, int jobs_per_group);   // the symmetric backprojection's dynamic shared memory
+size_t obp_smem_bytes(const ctr_plan *p);   // the symmetric backprojection's dynamic shared memory
+int obp_window(const std::vector<OrbitJob> &jobs, int nc);   // bins it stages per tile and job
+// p->ybar = g (N x M) in orbit layout: launch_backproject(p, (T *)p->ybar, ...) then reads it
+template <typename T> ctr_status launch_orbit_bar(const ctr_plan *p, const T *g, cudaStream_t s);
 void bp_tiles(int n, int &tx, int &ty);
 int fft_rows_per_cta(int n);
 bool wfft_supported(const ctr_plan *p);        // the warp-level preconditioner passes apply

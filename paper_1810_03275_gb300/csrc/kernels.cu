@@ -79,12 +79,13 @@ __device__ __forceinline__ void persist_stage_block(int stg, const SliceDesc *__
         return;
     }
     case BS_BP_SYM: {
+        if (tid >= OBP_THREADS) return;
         const int s = find_slice(pre, ns, vb);
         const SliceDesc &d = sd[s];
         const int local = vb - pre[s];
         const int bx = local % d.bp_tiles_x, rest = local / d.bp_tiles_x;
-        obp_body<float>(d.y1, d.n, d.M, d.wstride, d.per_group, d.n_jobs, d.jobs, d.bp_part, bx,
-                        rest % d.bp_tiles_y, rest / d.bp_tiles_y);
+        if (d.pair_jobs) obp_body<2, true>(obp_args(d), bx, rest % d.bp_tiles_y, rest / d.bp_tiles_y);
+        else obp_body<4, true>(obp_args(d), bx, rest % d.bp_tiles_y, rest / d.bp_tiles_y);
         return;
     }
     case BS_FFT_ROWS: {
@@ -163,7 +164,7 @@ k_batch_iteration(const SliceDesc *__restrict__ sd, const int *__restrict__ pref
                   unsigned long long spin_limit)
 {
     static_assert(32 * BP_TY <= PERSIST_THREADS && FWD_THREADS <= PERSIST_THREADS && ORBIT_THREADS <= PERSIST_THREADS &&
-                      32 * OBP_TY == PERSIST_THREADS && FFT_THREADS == PERSIST_THREADS,
+                      OBP_THREADS <= PERSIST_THREADS && FFT_THREADS == PERSIST_THREADS,
                   "stage bodies must fit the persistent CTA");
     constexpr int PHASES = 6;
     const int phase_stage[PHASES][2] = {{BS_BP, BS_BP_SYM}, {BS_FFT_ROWS, -1}, {BS_FFT_COLS, -1},

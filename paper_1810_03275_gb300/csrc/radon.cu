@@ -274,8 +274,22 @@ __device__ __forceinline__ T data_resolvent(T z, T s, T w, T a, T lo, T hi)
     return w * (z - s * a) / (s + w) + s * (q - fmin(fmax(q, lo), hi));
 }
 
+// The next iteration's backprojection operand: in orbit layout (ydst; rounded through
+// bfloat16 for a BF16 plan), in bfloat16, or as it is.
 template <typename T>
-__device__ __forceinline__ void forward_epilogue(const ForwardEpi<T> &epi, size_t r, T val)
+__device__ __forceinline__ void store_y1(const ForwardEpi<T> &epi, size_t r, T y, T *ydst)
+{
+    if constexpr (sizeof(T) == 4) {
+        if (ydst) *ydst = epi.yround ? __bfloat162float(__float2bfloat16_rn(y)) : y;
+        else if (epi.y1h) epi.y1h[r] = __float2bfloat16_rn(y);
+        else epi.y1[r] = y;
+    } else {
+        epi.y1[r] = y;
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void forward_epilogue(const ForwardEpi<T> &epi, size_t r, T val, T *ydst = nullptr)
 {
     if (epi.mode == 0) {
         epi.g[r] = val * epi.scale;
@@ -292,12 +306,7 @@ __device__ __forceinline__ void forward_epilogue(const ForwardEpi<T> &epi, size_
         const T Ru = val * epi.scale;
         const T y = Ru - epi.da[r];
         epi.Ru[r] = Ru;
-        if constexpr (sizeof(T) == 4) {
-            if (epi.y1h) epi.y1h[r] = __float2bfloat16_rn(y);
-            else epi.y1[r] = y;
-        } else {
-            epi.y1[r] = y;
-        }
+        store_y1(epi, r, y, ydst);
         if (epi.t1) epi.t1[r] = y;
         return;
     }
@@ -312,18 +321,13 @@ __device__ __forceinline__ void forward_epilogue(const ForwardEpi<T> &epi, size_
     const T vbn = vb + t - v1;
     epi.Ru[r] = Ru;
     epi.v1b[r] = vbn;
-    if constexpr (sizeof(T) == 4) {
-        if (epi.y1h) epi.y1h[r] = __float2bfloat16_rn(vbn + sigma * Ru);
-        else epi.y1[r] = vbn + sigma * Ru;
-    } else {
-        epi.y1[r] = vbn + sigma * Ru;
-    }
+    store_y1(epi, r, vbn + sigma * Ru, ydst);
     if (epi.t1) epi.t1[r] = t;
 }
 
 // The same epilogue (modes 1 and 2) on operands fetched ahead: vb = v1b[r], w, a, lo, hi.
 __device__ __forceinline__ void forward_epilogue_pre(const ForwardEpi<float> &epi, size_t r, float val, float vb,
-                                                     float w, float a, float lo, float hi)
+                                                     float w, float a, float lo, float hi, float *ydst)
 {
     const float sigma = epi.sigma;
     if (epi.mode == 2) {
@@ -338,8 +342,7 @@ __device__ __forceinline__ void forward_epilogue_pre(const ForwardEpi<float> &ep
     const float vbn = vb + t - v1;
     epi.Ru[r] = Ru;
     epi.v1b[r] = vbn;
-    if (epi.y1h) epi.y1h[r] = __float2bfloat16_rn(vbn + sigma * Ru);
-    else epi.y1[r] = vbn + sigma * Ru;
+    store_y1(epi, r, vbn + sigma * Ru, ydst);
     if (epi.t1) epi.t1[r] = t;
 }
 
@@ -843,14 +846,15 @@ __device__ __forceinline__ void march_orbit_rows(const L &ub, int n, long long K
     march_orbit<BPOS, true>(ub, n, mhi - ihi, r, q, off, A32, lim, B32, thr, Su, Sf);
 }
 
-__device__ __forceinline__ void orbit_out(const ForwardEpi<float> &epi, int l, int M, int k, int lane, float Su,
-                                          float Sf, const float *pre = nullptr)
+__device__ __forceinline__ void orbit_out(const ForwardEpi<float> &epi, int job, int c, int l, int M, int k, int lane,
+                                          float Su, float Sf, const float *pre = nullptr)
 {
     const float Bk = Sf - Su, Ak = Su - Bk;
     const float Bprev = __shfl_up_sync(0xffffffffu, Bk, 1);
     if (l >= 0 && lane >= 1 && k < M) {
-        if (pre) forward_epilogue_pre(epi, (size_t)l * M + k, Ak + Bprev, pre[0], pre[32], pre[64], pre[96], pre[128]);
-        else forward_epilogue(epi, (size_t)l * M + k, Ak + Bprev);
+        float *yd = epi.ybar ? epi.ybar + ((size_t)job * epi.ypitch + epi.ypad + k) * epi.ync + (c & (epi.ync - 1)) : nullptr;
+        if (pre) forward_epilogue_pre(epi, (size_t)l * M + k, Ak + Bprev, pre[0], pre[32], pre[64], pre[96], pre[128], yd);
+        else forward_epilogue(epi, (size_t)l * M + k, Ak + Bprev, yd);
     }
 }
 
@@ -885,9 +889,6 @@ constexpr int ORBIT_SLOTS = CTR_ORBIT_SLOTS;
 constexpr int ORBIT_THREADS = 32 * ORBIT_SLOTS * ORBIT_SEGS;
 #ifndef CTR_ORBIT_MINB
 #define CTR_ORBIT_MINB 8
-#endif
-#ifndef CTR_OBP_MINB
-#define CTR_OBP_MINB 4
 #endif
 
 // Warp w of the CTA takes job by*ORBIT_SLOTS + w % ORBIT_SLOTS, bins bx*31 + [0, 31) and
@@ -978,10 +979,10 @@ __device__ __forceinline__ void forward_orbit_body(const typename OrbitRec<S>::t
     if (!active) return;
     if (pre) cp_async_wait<0>();                      // this lane's own copies: no barrier needed
     const float *pe = pre ? s_epi[slot] + lane : nullptr;
-    orbit_out(epi, ls.x, M, k, lane, Su.x, Sf.x, pe ? pe + 0 * 160 : nullptr);
-    orbit_out(epi, ls.y, M, k, lane, Su.y, Sf.y, pe ? pe + 1 * 160 : nullptr);
-    orbit_out(epi, ls.z, M, k, lane, Su.z, Sf.z, pe ? pe + 2 * 160 : nullptr);
-    orbit_out(epi, ls.w, M, k, lane, Su.w, Sf.w, pe ? pe + 3 * 160 : nullptr);
+    orbit_out(epi, jb, 0, ls.x, M, k, lane, Su.x, Sf.x, pe ? pe + 0 * 160 : nullptr);
+    orbit_out(epi, jb, 1, ls.y, M, k, lane, Su.y, Sf.y, pe ? pe + 1 * 160 : nullptr);
+    orbit_out(epi, jb, 2, ls.z, M, k, lane, Su.z, Sf.z, pe ? pe + 2 * 160 : nullptr);
+    orbit_out(epi, jb, 3, ls.w, M, k, lane, Su.w, Sf.w, pe ? pe + 3 * 160 : nullptr);
 }
 
 // SLOTS adjacent jobs per CTA (their rays nearly coincide, so they share the orbit
@@ -1147,10 +1148,10 @@ k_forward_orbit_staged(const typename OrbitRec<S>::type *__restrict__ ubar, int 
     }
     cp_async_wait<0>();
     if (!has_job || kb >= M) return;             // warp-uniform
-    orbit_out(epi, ls.x, M, k, lane, Su.x, Sf.x);
-    orbit_out(epi, ls.y, M, k, lane, Su.y, Sf.y);
-    orbit_out(epi, ls.z, M, k, lane, Su.z, Sf.z);
-    orbit_out(epi, ls.w, M, k, lane, Su.w, Sf.w);
+    orbit_out(epi, j0 + warp, 0, ls.x, M, k, lane, Su.x, Sf.x);
+    orbit_out(epi, j0 + warp, 1, ls.y, M, k, lane, Su.y, Sf.y);
+    orbit_out(epi, j0 + warp, 2, ls.z, M, k, lane, Su.z, Sf.z);
+    orbit_out(epi, j0 + warp, 3, ls.w, M, k, lane, Su.w, Sf.w);
 }
 
 template <typename S>
@@ -1191,286 +1192,7 @@ void launch_forward_orbit(const ctr_plan *p, const typename OrbitRec<S>::type *u
     }
 }
 
-// ---------------------------------------------------------------------------
-// Symmetric backprojection (OrbitJob): a CTA owns a 32 x 32 tile of canonical
-// pixels x and a group of jobs; per job it stages the four channels' sinogram rows
-// side by side, so one fixed-point P(x) and one pair of 16-byte shared loads serve
-// four angles.  Channel v's sum at x belongs to image pixel T_v^{-1}(x); the four
-// channel images are written as partial planes [group][v][row][col] with
-//   plane 0 at x, plane 1 at x (its pixel is row-mirrored), planes 2 and 3 transposed
-// so that the fold reads rows only:
-//   u(i, j) = sum_groups P0[i][j] + P1[n-1-i][j] + P2[i][j] + P3[n-1-i][j].
-// ---------------------------------------------------------------------------
-#ifndef CTR_OBP_TY
-#define CTR_OBP_TY 8
-#endif
-#ifndef CTR_OBP_R
-#define CTR_OBP_R 4
-#endif
-constexpr int OBP_TY = CTR_OBP_TY;     // warps of a symmetric-backprojection CTA (32 x 32 tile)
-constexpr int OBP_R = CTR_OBP_R;       // pixels per thread (rows i0 + ty + OBP_TY r)
-#ifndef CTR_OBP_ASYNC
-#define CTR_OBP_ASYNC 1
-#endif
-constexpr bool OBP_ASYNC = CTR_OBP_ASYNC;
-#ifndef CTR_OBP_JCH
-#define CTR_OBP_JCH 8
-#endif
-constexpr int OBP_JCH = CTR_OBP_JCH;   // jobs per staged chunk (synchronous staging)
-#ifndef CTR_OBP_AJCH
-#define CTR_OBP_AJCH 24
-#endif
-constexpr int OBP_AJCH = CTR_OBP_AJCH; // jobs per staged chunk (asynchronous staging, two buffers)
-
-size_t obp_smem(int wstride, int jobs_per_group)
-{
-    // staged pairs + chunk tables (bfloat16 operands, synchronous staging) ...
-    const size_t stage = sizeof(float4) * 2 * OBP_JCH * wstride + (3 * sizeof(long long) + 5 * sizeof(int)) * OBP_JCH;
-    // ... or two raw chunk buffers + the whole group's tables (FP32, asynchronous staging)
-    const size_t async = sizeof(float4) * 2 * OBP_AJCH * (wstride + 1) +
-                         (3 * sizeof(long long) + 5 * sizeof(int)) * (size_t)jobs_per_group;
-    const size_t tr = sizeof(float) * 2 * 32 * 33;
-    return std::max(std::max(stage, async), tr);
-}
-
-// The FP32 symmetric backprojection with asynchronous staging: the group's job tables
-// are built once; chunk c + 1's four sinogram rows per job are copied raw into the
-// second of two shared buffers (cp.async, zero-filled outside the detector) while
-// chunk c is computed, so no global-load latency sits between chunks.  Each bin holds
-// the four channels' g as one float4; a (pixel, job) reads bins b and b + 1 and
-// interpolates g_b + f (g_{b+1} - g_b) per channel.
-template <bool PAIRS>
-__device__ __forceinline__ void obp_body_async(const float *__restrict__ g, int n, int M, int wstride,
-                                               int jobs_per_group, int n_jobs, const OrbitJob *__restrict__ jobs,
-                                               float (&acc)[OBP_R][4], int bx, int by, int bz)
-{
-    constexpr int NT = 32 * OBP_TY;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int WR = wstride + 1;                                           // bins per staged row
-    float4 *raw = reinterpret_cast<float4 *>(smem_raw);                   // [2][JCH][WR], channels in x..w
-    const int la = bz * jobs_per_group;
-    const int nj = max(0, min(n_jobs, la + jobs_per_group) - la);
-    // per job one 16-byte record {fraction of the tile's first P, S, C - 1, pair} (on the
-    // symmetric path 0 <= S < 2^32 and 1 <= C <= 2^32; pair = 1 or 2 for a job whose angles
-    // sit in channels {0, 1} or {2, 3} only, 0 otherwise): one shared load per warp and job
-    uint4 *sT = reinterpret_cast<uint4 *>(raw + 2 * OBP_AJCH * WR);
-    int *sK = reinterpret_cast<int *>(sT + jobs_per_group);
-    int *sL = sK + jobs_per_group;                                        // [job][channel]
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i0 = by * 32, j0 = bx * 32;
-    for (int t = threadIdx.x; t < nj; t += NT) {
-        const OrbitJob &jb = jobs[la + t];
-        const long long Cc = jb.am.A, Sc = jb.am.B;
-        const long long P00 = (long long)i0 * Cc + (long long)j0 * Sc + jb.am.Op;
-        const long long kmin = P00 >> 32;                                // Cc, Sc >= 0: the tile's minimum
-        sK[t] = (int)kmin;
-        const unsigned pair = !PAIRS ? 0u : (jb.l[2] < 0 && jb.l[3] < 0) ? 1u : ((jb.l[0] < 0 && jb.l[1] < 0) ? 2u : 0u);
-        sT[t] = make_uint4((unsigned)(P00 - (kmin << 32)), (unsigned)Sc, (unsigned)(Cc - 1), pair);
-        for (int c = 0; c < 4; ++c) sL[4 * t + c] = jb.l[c];
-    }
-    __syncthreads();
-    const int nch = (nj + OBP_AJCH - 1) / OBP_AJCH;
-    auto prefetch = [&](int ch) {
-        const int a0 = ch * OBP_AJCH, na = min(OBP_AJCH, nj - a0);
-        float *dst = reinterpret_cast<float *>(raw + (size_t)(ch & 1) * OBP_AJCH * WR);
-        // four-channel jobs: slot w = the four channels at bin k + w; pair jobs: slot w = the two
-        // live channels at bins k + w and k + w + 1 (lo and hi of one interpolation)
-        const unsigned mw = udiv_magic((unsigned)WR);
-        for (int e = threadIdx.x; e < na * WR * 4; e += NT) {
-            const int c = e & 3, rest = e >> 2;
-            const int a = udiv_fast(rest, WR, mw), w = rest - a * WR;
-            const unsigned pair = PAIRS ? sT[a0 + a].w : 0u;
-            const int ch = pair ? 2 * (int)(pair - 1) + (c & 1) : c;
-            const int k = sK[a0 + a] + w + (pair ? (c >> 1) : 0), l = sL[4 * (a0 + a) + ch];
-            const bool ok = l >= 0 && k >= 0 && k < M;
-            cp_async4(dst + (size_t)rest * 4 + c, ok ? g + (size_t)l * M + k : g, ok);
-        }
-    };
-    if (nch > 0) prefetch(0);
-    cp_async_commit();
-    for (int ch = 0; ch < nch; ++ch) {
-        if (ch + 1 < nch) prefetch(ch + 1);
-        cp_async_commit();
-        cp_async_wait<1>();                                               // this thread's copies of chunk ch
-        __syncthreads();                                                  // everyone's
-        const int a0 = ch * OBP_AJCH, na = min(OBP_AJCH, nj - a0);
-        const float4 *buf = raw + (size_t)(ch & 1) * OBP_AJCH * WR;
-#pragma unroll 2
-        for (int a = 0; a < na; ++a) {
-            const uint4 tj = sT[a0 + a];
-            const long long C = (long long)tj.z + 1;
-            long long P = (long long)tj.x + (long long)ty * C + (long long)tx * (long long)tj.y;
-            const long long D = C * OBP_TY;
-            const float4 *row = buf + a * WR;
-            if (PAIRS && tj.w) {                                          // pair job (CTA-uniform)
-                const bool p01 = tj.w == 1;
-#pragma unroll
-                for (int r = 0; r < OBP_R; ++r) {
-                    const int b = (int)(P >> 32);
-                    const float f = one_plus_frac32(P) - 1.f;
-                    const float4 v = row[b];                              // (lo, lo, hi, hi)
-                    const float2 lo = make_float2(v.x, v.y);
-                    const float2 t = ffma2(make_float2(f, f), fsub2(make_float2(v.z, v.w), lo), lo);
-                    if (p01) {
-                        const float2 s = fadd2(make_float2(acc[r][0], acc[r][1]), t);
-                        acc[r][0] = s.x;
-                        acc[r][1] = s.y;
-                    } else {
-                        const float2 s = fadd2(make_float2(acc[r][2], acc[r][3]), t);
-                        acc[r][2] = s.x;
-                        acc[r][3] = s.y;
-                    }
-                    P += D;
-                }
-                continue;
-            }
-#pragma unroll
-            for (int r = 0; r < OBP_R; ++r) {
-                const int b = (int)(P >> 32);
-                const float f = one_plus_frac32(P) - 1.f;                 // exact: the 23 fraction bits
-                const float4 lo = row[b], hi = row[b + 1];
-                const float2 f2 = make_float2(f, f);
-                const float2 lo01 = make_float2(lo.x, lo.y), lo23 = make_float2(lo.z, lo.w);
-                const float2 t01 = ffma2(f2, fsub2(make_float2(hi.x, hi.y), lo01), lo01);
-                const float2 t23 = ffma2(f2, fsub2(make_float2(hi.z, hi.w), lo23), lo23);
-                const float2 a01 = fadd2(make_float2(acc[r][0], acc[r][1]), t01);
-                const float2 a23 = fadd2(make_float2(acc[r][2], acc[r][3]), t23);
-                acc[r][0] = a01.x;
-                acc[r][1] = a01.y;
-                acc[r][2] = a23.x;
-                acc[r][3] = a23.y;
-                P += D;
-            }
-        }
-        __syncthreads();                                                  // buffer ch & 1 is refilled next
-    }
-    cp_async_wait<0>();
-}
-
-template <typename S, bool PAIRS = false>
-__device__ __forceinline__ void obp_body(const S *__restrict__ g, int n, int M, int wstride, int jobs_per_group,
-                                         int n_jobs, const OrbitJob *__restrict__ jobs, float *__restrict__ part,
-                                         int bx, int by, int bz)
-{
-    static_assert(OBP_TY * OBP_R == 32, "32 x 32 tiles");
-    constexpr int NT = 32 * OBP_TY;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *stage = reinterpret_cast<float4 *>(smem_raw);               // [job][channel pair][bin]
-    long long *sPb = reinterpret_cast<long long *>(stage + 2 * OBP_JCH * wstride);
-    long long *sC = sPb + OBP_JCH;
-    long long *sS = sC + OBP_JCH;
-    int *sK = reinterpret_cast<int *>(sS + OBP_JCH);
-    int *sL = sK + OBP_JCH;                                               // [job][channel]
-
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int i0 = by * 32, j0 = bx * 32;
-    const int la = bz * jobs_per_group;
-    const int lb = min(n_jobs, la + jobs_per_group);
-    float acc[OBP_R][4];
-#pragma unroll
-    for (int r = 0; r < OBP_R; ++r) acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f;
-
-    if constexpr (sizeof(S) == 4 && OBP_ASYNC)
-        obp_body_async<PAIRS>(g, n, M, wstride, jobs_per_group, n_jobs, jobs, acc, bx, by, bz);
-    else
-    for (int c0 = la; c0 < lb; c0 += OBP_JCH) {
-        const int na = min(OBP_JCH, lb - c0);
-        __syncthreads();
-        if (threadIdx.x < na) {
-            const AngleMarch am = jobs[c0 + threadIdx.x].am;     // canonical P(i, j) = i A + j B + Op
-            const long long Cc = am.A, Sc = am.B;
-            const long long P00 = (long long)i0 * Cc + (long long)j0 * Sc + am.Op;
-            const long long kmin = P00 >> 32;                    // Cc, Sc >= 0: P00 is the tile's minimum
-            sK[threadIdx.x] = (int)kmin;
-            sPb[threadIdx.x] = P00 - (kmin << 32);
-            sC[threadIdx.x] = Cc;
-            sS[threadIdx.x] = Sc;
-        }
-        if (threadIdx.x < 4 * na) sL[threadIdx.x] = jobs[c0 + (threadIdx.x >> 2)].l[threadIdx.x & 3];
-        __syncthreads();
-        float *stf = reinterpret_cast<float *>(stage);
-        const unsigned mw = udiv_magic((unsigned)wstride);
-        for (int e = threadIdx.x; e < na * wstride * 4; e += NT) {
-            const int c = e & 3, rest = e >> 2;
-            const int a = udiv_fast(rest, wstride, mw), w = rest - a * wstride;
-            const int k = sK[a] + w, l = sL[4 * a + c];
-            const S *row = g + (size_t)(l < 0 ? 0 : l) * M;
-            const float g0 = (l >= 0 && k >= 0 && k < M) ? ldv(row + k) : 0.f;
-            const float g1 = (l >= 0 && k + 1 >= 0 && k + 1 < M) ? ldv(row + k + 1) : 0.f;
-            // float4 planes (ch0 ch1) and (ch2 ch3) of the job, consecutive bins adjacent; in
-            // each float4 the two channels' (g0 - d) first, then their d = g1 - g0
-            const float2 st = make_stage(g0, g1);
-            float *q = stf + ((size_t)(2 * a + (c >> 1)) * wstride + w) * 4 + (c & 1);
-            q[0] = st.x;
-            q[2] = st.y;
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int a = 0; a < na; ++a) {
-            const long long C = sC[a];
-            long long P = sPb[a] + (long long)ty * C + (long long)tx * sS[a];
-            const long long D = C * OBP_TY;
-            const float4 *row01 = stage + 2 * a * wstride;
-            const float4 *row23 = row01 + wstride;
-#pragma unroll
-            for (int r = 0; r < OBP_R; ++r) {
-                const int b = (int)(P >> 32);
-                const float f = one_plus_frac32(P);
-                const float4 s01 = row01[b], s23 = row23[b];
-                const float2 f2 = make_float2(f, f);
-                const float2 a01 = ffma2(f2, make_float2(s01.z, s01.w),
-                                         fadd2(make_float2(acc[r][0], acc[r][1]), make_float2(s01.x, s01.y)));
-                const float2 a23 = ffma2(f2, make_float2(s23.z, s23.w),
-                                         fadd2(make_float2(acc[r][2], acc[r][3]), make_float2(s23.x, s23.y)));
-                acc[r][0] = a01.x;
-                acc[r][1] = a01.y;
-                acc[r][2] = a23.x;
-                acc[r][3] = a23.y;
-                P += D;
-            }
-        }
-    }
-
-    const size_t nn = (size_t)n * n;
-    float *pg = part + (size_t)bz * 4 * nn;
-    const int j = j0 + tx;
-#pragma unroll
-    for (int r = 0; r < OBP_R; ++r) {
-        const int i = i0 + ty + OBP_TY * r;
-        if (i < n && j < n) {
-            pg[(size_t)i * n + j] = acc[r][0];
-            pg[nn + (size_t)i * n + j] = acc[r][1];
-        }
-    }
-    // planes 2 and 3 transposed through shared memory (coalesced rows j)
-    __syncthreads();
-    float(*tr)[32][33] = reinterpret_cast<float(*)[32][33]>(smem_raw);
-#pragma unroll
-    for (int r = 0; r < OBP_R; ++r) {
-        tr[0][ty + OBP_TY * r][tx] = acc[r][2];
-        tr[1][ty + OBP_TY * r][tx] = acc[r][3];
-    }
-    __syncthreads();
-    const int it = i0 + tx;
-#pragma unroll
-    for (int r = 0; r < OBP_R; ++r) {
-        const int jl = ty + OBP_TY * r, jt = j0 + jl;
-        if (it < n && jt < n) {
-            pg[2 * nn + (size_t)jt * n + it] = tr[0][tx][jl];
-            pg[3 * nn + (size_t)jt * n + it] = tr[1][tx][jl];
-        }
-    }
-}
-
-template <typename S, bool PAIRS>
-__global__ void __launch_bounds__(32 * OBP_TY, CTR_OBP_MINB)
-k_backproject_orbit(const S *__restrict__ g, int n, int M, int wstride, int jobs_per_group, int n_jobs,
-                    const OrbitJob *__restrict__ jobs, float *__restrict__ part)
-{
-    pdl_wait();
-    pdl_trigger();
-    obp_body<S, PAIRS>(g, n, M, wstride, jobs_per_group, n_jobs, jobs, part, blockIdx.x, blockIdx.y, blockIdx.z);
-}
+#include "orbit.cuh"
 
 // The fold of the symmetric backprojection's partial planes, then the
 // backprojection epilogue (grid-stride over the pixels).
@@ -1511,7 +1233,13 @@ k_backproject_batch(const SliceDesc *__restrict__ sd, const int *__restrict__ pr
                           d.bp_groups > 1 ? d.bp_part : nullptr, bx, by, bz);
 }
 
-__global__ void __launch_bounds__(32 * OBP_TY, CTR_OBP_MINB)
+__device__ __forceinline__ ObpArgs obp_args(const SliceDesc &d)
+{
+    return ObpArgs{d.ybar, d.jobs, d.bp_part, d.n, d.bar_pitch, d.bar_pad, d.obp_win, d.bp_groups,
+                   {d.job_list[0], d.job_list[1], d.job_list[2]}};
+}
+
+__global__ void __launch_bounds__(OBP_THREADS, 4)
 k_backproject_orbit_batch(const SliceDesc *__restrict__ sd, const int *__restrict__ prefix, int ns)
 {
     const int s = find_slice(prefix, ns, blockIdx.x);
@@ -1519,8 +1247,8 @@ k_backproject_orbit_batch(const SliceDesc *__restrict__ sd, const int *__restric
     const int local = blockIdx.x - prefix[s];
     const int bx = local % d.bp_tiles_x, rest = local / d.bp_tiles_x;
     const int by = rest % d.bp_tiles_y, bz = rest / d.bp_tiles_y;
-    if (d.pair_jobs) obp_body<float, true>(d.y1, d.n, d.M, d.wstride, d.per_group, d.n_jobs, d.jobs, d.bp_part, bx, by, bz);
-    else obp_body<float, false>(d.y1, d.n, d.M, d.wstride, d.per_group, d.n_jobs, d.jobs, d.bp_part, bx, by, bz);
+    if (d.pair_jobs) obp_body<2, false>(obp_args(d), bx, by, bz);
+    else obp_body<4, false>(obp_args(d), bx, by, bz);
 }
 
 __global__ void __launch_bounds__(256)
@@ -1584,21 +1312,37 @@ void launch_fwd_cfg(const ctr_plan *p, dim3 grid, const S *u, const S *uT, const
     k_forward<T, S, NC, EXACT1><<<grid, FWD_THREADS, 0, s>>>(u, uT, p->n, p->N, p->M, p->F, p->d_march, epi);
 }
 
+// g (N x M) into orbit layout (bar)
+template <typename S>
+ctr_status launch_orbit_sino(const ctr_plan *p, const S *g, float *bar, cudaStream_t s)
+{
+    p->launches++;
+    const dim3 grid((p->M + 255) / 256, p->n_jobs);
+    auto kern = p->pair_jobs ? k_orbit_sino<S, 2> : k_orbit_sino<S, 4>;
+    launch_pdl(p->pdl != 0, kern, grid, dim3(256), 0, s, g, p->M, p->n_jobs, p->job_list[1], p->bar_pitch, p->bar_pad,
+               (const OrbitJob *)p->d_jobs, bar);
+    CTR_CHECK_LAUNCH("k_orbit_sino");
+    return CTR_OK;
+}
+
 template <typename T, typename S>
 ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cudaStream_t s, bool defer_reduce)
 {
     if constexpr (sizeof(T) == 4) {
         if (p->orbit) {
             const int G = p->obp_groups;
-            dim3 grid((p->n + BP_TJ - 1) / BP_TJ, (p->n + BP_TI - 1) / BP_TI, G);
+            const dim3 grid((p->n + 31) / 32, (p->n + 31) / 32, G);
             float *part = (float *)p->obp_part;
+            const float *bar = (const float *)p->ybar;
+            if ((const void *)g != p->ybar) {                              // an operand in sinogram layout
+                ctr_status st = launch_orbit_sino<S>(p, g, (float *)p->gbar, s);
+                if (st != CTR_OK) return st;
+                bar = (const float *)p->gbar;
+            }
             p->launches++;
-            const int jpg = (p->n_jobs + G - 1) / G;
-            auto kern = k_backproject_orbit<S, false>;
-            if constexpr (sizeof(S) == 4)                                 // pair-job variant: FP32 staging only
-                if (p->pair_jobs) kern = k_backproject_orbit<S, true>;
-            launch_pdl(p->pdl != 0, kern, grid, dim3(32 * OBP_TY), obp_smem(p->wstride, jpg), s,
-                       g, p->n, p->M, p->wstride, jpg, p->n_jobs, (const OrbitJob *)p->d_jobs, part);
+            auto kern = p->pair_jobs ? k_backproject_orbit<2> : k_backproject_orbit<4>;
+            launch_pdl(p->pdl != 0, kern, grid, dim3(OBP_THREADS), obp_smem(p->obp_win, p->pair_jobs ? 2 : 4), s,
+                       obp_args(p, bar));
             CTR_CHECK_LAUNCH("k_backproject_orbit");
             if (!defer_reduce) {
                 const size_t nn = (size_t)p->n * p->n;
@@ -1678,10 +1422,9 @@ ctr_status configure_radon(const ctr_plan *p)
 {
     const size_t smem = bp_smem<T>(p);
     ctr_status st = raise_smem_limit(k_backproject<T, T>, smem);
-    const size_t osm = p->orbit ? obp_smem(p->wstride, p->n_jobs) : 0;   // any group split
-    if (st == CTR_OK && p->orbit) st = raise_smem_limit(k_backproject_orbit<float, false>, osm);
-    if (st == CTR_OK && p->orbit) st = raise_smem_limit(k_backproject_orbit<float, true>, osm);
-    if (st == CTR_OK && p->orbit) st = raise_smem_limit(k_backproject_orbit<__nv_bfloat16, false>, osm);
+    if (st == CTR_OK && p->orbit)
+        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2>, obp_smem(p->obp_win, 2))
+                          : raise_smem_limit(k_backproject_orbit<4>, obp_smem(p->obp_win, 4));
     if constexpr (sizeof(T) == 4)
         if (st == CTR_OK) st = raise_smem_limit(k_backproject<float, __nv_bfloat16>, smem);
     if (st == CTR_OK && p->orbit && p->stg_wmax > 0) {
@@ -1778,7 +1521,25 @@ int stg_window(const std::vector<OrbitJob> &jobs, int n, int M)
 int orbit_fwd_grid_y(int n_jobs) { return (n_jobs + ORBIT_SLOTS - 1) / ORBIT_SLOTS; }
 int fwd_grid_y(int N) { return (N + FWD_AW - 1) / FWD_AW; }
 
-size_t obp_smem_bytes(int wstride, int jobs_per_group) { return obp_smem(wstride, jobs_per_group); }
+size_t obp_smem_bytes(const ctr_plan *p) { return obp_smem(p->obp_win, p->pair_jobs ? 2 : 4); }
+
+int obp_window(const std::vector<OrbitJob> &jobs, int nc)
+{
+    // bins of a tile's block centres (30 C + 28 S), two on the left and three on the right,
+    // and what the 16-byte alignment of the first bin adds
+    const int al = 4 / nc;
+    long long w = 0;
+    for (const OrbitJob &j : jobs) w = std::max(w, (30 * j.am.A + 28 * j.am.B) >> 32);
+    return ((int)w + 7 + (al - 1) + al - 1) & ~(al - 1);
+}
+
+template <typename T>
+ctr_status launch_orbit_bar(const ctr_plan *p, const T *g, cudaStream_t s)
+{
+    return launch_orbit_sino<T>(p, g, (float *)p->ybar, s);
+}
+template ctr_status launch_orbit_bar<float>(const ctr_plan *, const float *, cudaStream_t);
+template ctr_status launch_orbit_bar<__nv_bfloat16>(const ctr_plan *, const __nv_bfloat16 *, cudaStream_t);
 
 size_t bp_smem_bytes(int wstride)
 {
@@ -1805,7 +1566,7 @@ ctr_status launch_batch_radon(int stage, const SliceDesc *sd, const int *prefix,
     if (blocks <= 0) return CTR_OK;
     switch (stage) {
     case BS_BP: k_backproject_batch<<<blocks, 32 * BP_TY, smem, s>>>(sd, prefix, ns); break;
-    case BS_BP_SYM: k_backproject_orbit_batch<<<blocks, 32 * OBP_TY, smem, s>>>(sd, prefix, ns); break;
+    case BS_BP_SYM: k_backproject_orbit_batch<<<blocks, OBP_THREADS, smem, s>>>(sd, prefix, ns); break;
     case BS_ORBIT: k_orbit_image_batch<<<blocks, 256, 0, s>>>(sd, prefix, ns); break;
     case BS_FWD_SYM: k_forward_orbit_batch<<<blocks, ORBIT_THREADS, 0, s>>>(sd, prefix, ns); break;
     case BS_FWD: k_forward_batch<<<blocks, FWD_THREADS, 0, s>>>(sd, prefix, ns); break;

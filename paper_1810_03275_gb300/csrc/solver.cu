@@ -666,6 +666,17 @@ struct IterArgs {
     bool alg3 = false;     // Alg. 3: data term in the quadratic part, only the TV term dualised
 };
 
+// The forward epilogue writes the next y1 in orbit layout (symmetric path).
+template <typename T>
+void set_ybar(const ctr_plan *p, ForwardEpi<T> &e)
+{
+    e.ybar = (T *)p->ybar;
+    e.ypitch = p->bar_pitch;
+    e.ypad = p->bar_pad;
+    e.ync = p->pair_jobs ? 2 : 4;
+    e.yround = p->bf16 ? 1 : 0;
+}
+
 // One iteration of Alg. 4 (steps A-D).  diag: also keep du, t1, t2 for diagnostics.
 template <typename T>
 ctr_status pdrq_iteration(ctr_plan *p, const IterArgs<T> &a, bool diag, cudaStream_t s)
@@ -688,9 +699,12 @@ ctr_status pdrq_iteration(ctr_plan *p, const IterArgs<T> &a, bool diag, cudaStre
     }
     const bool h = sizeof(T) == 4 && p->bf16;   // projector operands in bfloat16
     const bool fuse = bp_deferred<T>(p);        // partial-image sum and epilogue inside the first FFT pass
-    if (h) {
+    const bool bar = sizeof(T) == 4 && p->orbit;   // symmetric path: y1 is kept in orbit layout
+    if (h && !bar) {
         if constexpr (sizeof(T) == 4)
             if ((st = launch_backproject_bf16(p, p->y1h, ea, s, fuse)) != CTR_OK) return st;
+    } else if (bar) {
+        if ((st = launch_backproject<T>(p, (const T *)p->ybar, ea, s, fuse)) != CTR_OK) return st;
     } else if ((st = launch_backproject<T>(p, (const T *)p->y1, ea, s, fuse)) != CTR_OK) {
         return st;
     }
@@ -709,6 +723,7 @@ ctr_status pdrq_iteration(ctr_plan *p, const IterArgs<T> &a, bool diag, cudaStre
     ec.Ru = (T *)p->Ru;
     ec.v1b = (T *)p->v1b;
     ec.y1 = (T *)p->y1;
+    if (bar) set_ybar<T>(p, ec);
     ec.t1 = diag ? (T *)p->t1 : nullptr;
     const T *d = (const T *)p->desc;
     ec.dw = d;
@@ -1237,6 +1252,11 @@ ctr_status pdrq_loop(ctr_plan *p, double alpha, int iters, const ctr_params &prm
         p->launches++;
         k_to_bf16<<<grid_for(nm, 256, 4096), 256, 0, s>>>((const float *)p->y1, nm, p->y1h);
     }
+    if constexpr (sizeof(T) == 4) {
+        if (p->orbit && (st = p->bf16 ? launch_orbit_bar(p, (const __nv_bfloat16 *)p->y1h, s)
+                                      : launch_orbit_bar(p, (const float *)p->y1, s)) != CTR_OK)
+            return st;
+    }
     CTR_CHECK_LAUNCH("pdrq init");
     if (iters <= 0) {
         CTR_CUDA(cudaMemsetAsync(p->du, 0, nn * sizeof(T), s));
@@ -1554,6 +1574,7 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         k_init_y2<float><<<grid_for(nn, 256, 4096), 256, 0, s>>>((const float *)p->u, (const float *)p->v2b, p->n,
                                                                a.sigma * a.tau, a.inv_h, (float *)p->y2);
         CTR_CHECK_LAUNCH("batch init");
+        if (p->orbit && (st = launch_orbit_bar(p, (const float *)p->y1, s)) != CTR_OK) return st;
         SliceDesc &d = hd[i];
         d.n = p->n;
         d.N = p->N;
@@ -1565,6 +1586,11 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.n_jobs = p->n_jobs;
         d.jobs = p->d_jobs;
         d.ubar = (float4 *)p->ubar;
+        d.ybar = (const float *)p->ybar;
+        d.bar_pitch = p->bar_pitch;
+        d.bar_pad = p->bar_pad;
+        d.obp_win = p->obp_win;
+        for (int k = 0; k < 3; ++k) d.job_list[k] = p->job_list[k];
         d.bp_groups = p->orbit ? p->obp_groups : p->bp_groups;
         d.per_group = p->orbit ? (p->n_jobs + p->obp_groups - 1) / p->obp_groups
                                : (p->N + p->bp_groups - 1) / p->bp_groups;
@@ -1608,6 +1634,7 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.fwe.Ru = (float *)p->Ru;
         d.fwe.v1b = (float *)p->v1b;
         d.fwe.y1 = (float *)p->y1;
+        if (p->orbit) set_ybar<float>(p, d.fwe);
         const float *dd = (const float *)p->desc;
         d.fwe.dw = dd;
         d.fwe.da = dd + nm;
@@ -1716,7 +1743,7 @@ ctr_status batch_prepare(ctr_batch *b)
         cnt[BS_FWD_SYM] = p->orbit ? fwd_grid_x(p->M) * orbit_fwd_grid_y(p->n_jobs) : 0;
         cnt[BS_TV] = grid_for(nn, 256, 1024);
         for (int stg = 0; stg < BS_COUNT; ++stg) pre[(size_t)stg * (ns + 1) + i + 1] = pre[(size_t)stg * (ns + 1) + i] + cnt[stg];
-        const size_t smb = p->orbit ? 0 : bp_smem_bytes(p->wstride), smo = p->orbit ? obp_smem_bytes(p->wstride, (p->n_jobs + p->obp_groups - 1) / p->obp_groups) : 0;
+        const size_t smb = p->orbit ? 0 : bp_smem_bytes(p->wstride), smo = p->orbit ? obp_smem_bytes(p) : 0;
         if (smo > b->smem[BS_BP_SYM]) b->smem[BS_BP_SYM] = smo;
         const size_t smr = packed ? fft_packed_smem(p, 0) : fft_rows_smem(p->n, sizeof(float));
         const size_t smc = packed ? fft_packed_smem(p, 1) : fft_cols_smem(p->n, sizeof(float));
