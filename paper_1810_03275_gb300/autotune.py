@@ -67,8 +67,8 @@ def _time(fn, reps: int) -> float:
 
 
 def _try_shape(plan, shape) -> bool:
-    """Set a forward launch shape; False where the plan does not offer it (the staged
-    shape needs its orbit-image window to fit one CTA's shared memory)."""
+    """Set a forward launch shape; False where the plan does not offer it ((4, 1) needs the
+    rays of four adjacent jobs to be close)."""
     from . import ctrecon as ct
     try:
         plan.set_fwd_shape(*shape)

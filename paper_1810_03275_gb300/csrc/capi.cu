@@ -114,6 +114,32 @@ long long floor_div2(__int128 v)
 // its canonical pair a = max(|C|, |S|), b = min(|C|, |S|) (true for angles in
 // [0, pi)); angles with equal canonical pairs share a job, one per channel.  The
 // path is taken when the jobs hold two angles or more on average.
+// Whether ctr_plan_set_fwd_shape takes (4, 1): two blocks of 8 rows of the pixels that four
+// consecutive jobs (in the order of their first angles) cross must fit one CTA's shared memory.
+bool shape41_fits(const std::vector<OrbitJob> &jobs, int n, int M)
+{
+    const double one = 4294967296.0;
+    double w = 0.0;
+    for (size_t g = 0; g < jobs.size(); g += 4) {
+        const size_t e = std::min(jobs.size(), g + 4);
+        double spread = 0.0, span = 0.0;
+        for (double K : {-one, (double)(M + 32) * one})
+            for (double m : {0.0, (double)(n - 1)}) {
+                double lo = 1e300, hi = -1e300;
+                for (size_t j = g; j < e; ++j) {
+                    const double x = (K - m * (double)jobs[j].am.B - (double)jobs[j].am.Op) / (double)jobs[j].am.A;
+                    lo = std::min(lo, x);
+                    hi = std::max(hi, x);
+                }
+                spread = std::max(spread, hi - lo);
+            }
+        for (size_t j = g; j < e; ++j)
+            span = std::max(span, (32.0 * one + 7 * (double)jobs[j].am.B) / (double)jobs[j].am.A);
+        w = std::max(w, std::ceil(spread + span) + 4.0);
+    }
+    return 2.0 * 8 * std::floor(w) * 16 + 2.0 * sizeof(int) * ((n + 8) / 8 + 1) <= 227 * 1024;
+}
+
 ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
 {
     const int n = p->n, N = p->N, M = p->M;
@@ -168,6 +194,7 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
             if ((jb.l[2] < 0 && jb.l[3] < 0) || (jb.l[0] < 0 && jb.l[1] < 0)) ++pairs;
         p->pair_jobs = 2 * pairs > jobs.size() ? 1 : 0;
     }
+    p->shape41 = shape41_fits(jobs, n, M);
     // the job lists: one, or the pair jobs of channels {0, 1} and those of {2, 3} (a job with
     // angles in both becomes two); each sorted by S / C, so that neighbours' rays nearly coincide
     {
@@ -194,7 +221,7 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     const int nc = p->pair_jobs ? 2 : 4;
     {
         // orbit-layout rows: every tile's window of obp_win bins, and the detector, inside the row
-        p->obp_win = obp_window(jobs, nc);
+        p->obp_win = obp_window(jobs);
         const long long far = (n + 31) / 32 * 32 - 32;             // origin of the last tile
         long long lo = 0, hi = M;
         for (const OrbitJob &jb : jobs) {
@@ -209,8 +236,9 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     void *tmp = nullptr;
     if ((st = alloc(p, &tmp, sizeof(OrbitJob) * jobs.size())) != CTR_OK) return st;
     p->d_jobs = (OrbitJob *)tmp;
-    if ((st = alloc(p, &p->ubar, sizeof(float4) * (size_t)n * n)) != CTR_OK) return st;
-    // (the orbit image holds FP32 records; a BF16 plan's bfloat16 records use its first half)
+    if ((st = alloc(p, &p->ubar, sizeof(float4) * (size_t)n * orbit_pitch(n))) != CTR_OK) return st;
+    CTR_CUDA(cudaMemset(p->ubar, 0, sizeof(float4) * (size_t)n * orbit_pitch(n)));   // the pads stay zero
+    p->fwd_chunks = orbit_fwd_chunks(jobs, M);
     // the symmetric backprojection: job groups so that tiles x groups is about 1024 CTAs
     // (~1.7 waves of 4 eight-warp CTAs per SM on 152 SMs; measured best at n = 512 among
     // 2..8), at least 8 jobs per group; room for up to MAX_BP_GROUPS groups at n <= 1024
@@ -231,11 +259,6 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     CTR_CUDA(cudaMemcpy(p->d_jobs, jobs.data(), sizeof(OrbitJob) * jobs.size(), cudaMemcpyHostToDevice));
     p->n_jobs = (int)jobs.size();
     p->orbit = true;
-    // the staged forward shape only where its double-buffered window fits one CTA's shared
-    // memory (stg_wmax = 0: shape (4, 1) unavailable on this plan)
-    p->stg_wmax = stg_window(jobs, n, M);
-    p->stg_nst = stg_blocks_max(n);
-    if (stg_smem_bytes(p->stg_wmax, p->stg_nst, 16) > STG_SMEM_LIMIT) p->stg_wmax = 0;
     return CTR_OK;
 }
 
@@ -1016,9 +1039,9 @@ ctr_status ctr_plan_set_fwd_shape(ctr_plan *p, int jobs_per_cta, int segments)
         key != 4 * 16 + 2 && key != 4 * 16 + 1)
         return fail(CTR_EINVAL, "forward shape must be (1, 2), (1, 4), (1, 8), (2, 2), (2, 4), (4, 2) or (4, 1)");
     if (!p->orbit) return fail(CTR_EUNSUPPORTED, "the plan projects angle by angle (no symmetric forward projector)");
-    if (key == 4 * 16 + 1 && p->stg_wmax <= 0)
-        return fail(CTR_EUNSUPPORTED, "the staged forward shape (4, 1): its orbit-image window exceeds shared memory "
-                                      "on this geometry");
+    if (key == 4 * 16 + 1 && !p->shape41)
+        return fail(CTR_EUNSUPPORTED, "the forward shape (4, 1): the rays of four adjacent jobs are too far apart on "
+                                      "this geometry");
     p->fwd_slots = jobs_per_cta;
     p->fwd_segs = segments;
     return CTR_OK;

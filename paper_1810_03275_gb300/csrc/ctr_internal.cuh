@@ -77,10 +77,13 @@ inline cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim
 // whole process, shared by every plan: only ever raise it.  (Its default is 48 KB minus
 // the kernel's static shared memory, so the check is against the attribute itself.)
 template <typename K>
-inline ctr_status raise_smem_limit(K *kernel, size_t bytes)
+inline ctr_status raise_smem_limit(K *kernel, size_t bytes, bool full_carveout = false)
 {
     cudaFuncAttributes a;
     CTR_CUDA(cudaFuncGetAttributes(&a, (const void *)kernel));
+    if (full_carveout)
+        CTR_CUDA(cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      cudaSharedmemCarveoutMaxShared));
     if ((size_t)a.maxDynamicSharedSizeBytes >= bytes) return CTR_OK;
     CTR_CUDA(cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
     return CTR_OK;
@@ -281,7 +284,7 @@ struct ForwardEpi {
     T *y1;             // out: bar v1_new + sigma Rt u_new
     __nv_bfloat16 *y1h;   // if set: y1 is stored here in bfloat16 instead (BF16 operand storage)
     T *ybar;           // if set (symmetric path): y1 is stored here in orbit layout instead ...
-    int ypitch, ypad, ync;   // ... rows of ypitch bins of ync channels, bin 0 at ypad
+    int ypitch, ypad;  // ... rows of ypitch bins, bin 0 at ypad
     int yround;        // ... rounded through bfloat16 (BF16 plans)
     T *t1;             // optional out: resolvent output (dual certificate)
     const T *dw, *da, *dlo, *dhi;   // per-bin data term, beta-scaled
@@ -313,7 +316,7 @@ struct SliceDesc {
     float *ub;                    // Alg. 5: bar u (updated by the TV stage); null for Alg. 4
     int n_jobs;
     const OrbitJob *jobs;
-    float4 *ubar;
+    float *ubar;
     const float *ybar;            // the backprojection's operand in orbit layout ...
     int bar_pitch, bar_pad, obp_win, job_list[3];   // ... its shape and job lists (see ctr_plan)
     BackprojEpi<float> bpe;       // step A epilogue
@@ -400,12 +403,14 @@ struct ctr_plan {
     bool orbit = false;                  // FP32 forward projector on the symmetric path
     int n_jobs = 0;
     ctr::OrbitJob *d_jobs = nullptr;
-    void *ubar = nullptr;                // n*n float4 orbit image
+    void *ubar = nullptr;                // orbit image: two planes of n rows of orbit_pitch pixels, 8 bytes each
+    int fwd_chunks = 1;                  // symmetric forward projector: chunks of bins per job, at most
     int obp_groups = 1;                  // job groups of the symmetric backprojection
     int pair_jobs = 0;                   // most jobs are pair jobs: both projectors take their pair variants
     int obp_cap = 1;                     // groups the partial-plane workspace has room for
-    // sinogram operands of the symmetric backprojection in orbit layout: one row per job,
-    // bar_pitch bins of 4 (pair plans: 2) channels, bin 0 at bar_pad, zeros around the detector
+    // sinogram operands of the symmetric backprojection in orbit layout: per job a row of
+    // channels {0, 1} and one of {2, 3} (pair plans: one row), bar_pitch bins, bin 0 at bar_pad,
+    // zeros around the detector
     void *gbar = nullptr;                // operand of a single call
     void *ybar = nullptr;                // the iteration's y1, written by the forward epilogue
     int bar_pitch = 0, bar_pad = 0;
@@ -459,8 +464,7 @@ struct ctr_plan {
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     int fwd_slots = 1;                   // symmetric forward projector: adjacent jobs per CTA (1, 2, 4) ...
     int fwd_segs = 4;                    // ... and warps splitting a job's rows (2, 4, 8); see ctr_plan_set_fwd_shape
-    int stg_wmax = 0;                    // staged forward shape (4, 1): widest window (pixels) ...
-    int stg_nst = 0;                     // ... and most row blocks of one CTA
+    bool shape41 = false;                // ctr_plan_set_fwd_shape takes (4, 1)
     double *d_hist = nullptr;            // MAX_CHECKS x HIST_FIELDS diagnostics records
     int hist_count = 0;                  // records the last solve wrote
     ctr::GraphCache graphs;              // instantiated iteration graphs, reused across calls
@@ -522,17 +526,18 @@ template <typename T> bool bp_deferred(const ctr_plan *p);
 // orbit image): callers may then skip making the transposed copy uT
 template <typename T> inline bool fwd_needs_transpose(const ctr_plan *p) { return !(sizeof(T) == 4 && p->orbit); }
 int fwd_grid_x(int M);         // forward-projector grid: bin chunks
-size_t stg_smem_bytes(int wmax, int nst_max, int rec_bytes);   // the staged forward projector's shared memory
-constexpr size_t STG_SMEM_LIMIT = 227 * 1024;                   // dynamic shared memory one CTA may opt into
-int stg_blocks_max(int n);
-int stg_window(const std::vector<OrbitJob> &jobs, int n, int M);
-int orbit_fwd_grid_y(int n_jobs);   // symmetric forward projector: job groups per bin chunk
+int ofw_batch_groups(const ctr_plan *p);        // symmetric forward projector, batched stage: groups of jobs
+int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M);   // symmetric forward projector: bin chunks per job
+// its pixels per warp and row, and the zero pixels on either side of an orbit-image row (every
+// read of the march lies within them)
+constexpr int OFW_LANES = 64, ORBIT_PAD = OFW_LANES + 8;
+__host__ __device__ constexpr int orbit_pitch(int n) { return (n + 2 * ORBIT_PAD + 1) / 2 * 2; }
 int fwd_grid_y(int N);         // forward-projector grid: angle groups
 
 // batched stages (one launch per stage over all slices of a batch)
 size_t bp_smem_bytes(int wstride);
 size_t obp_smem_bytes(const ctr_plan *p);   // the symmetric backprojection's dynamic shared memory
-int obp_window(const std::vector<OrbitJob> &jobs, int nc);   // bins it stages per tile and job
+int obp_window(const std::vector<OrbitJob> &jobs);   // bins it stages per tile and job
 // p->ybar = g (N x M) in orbit layout: launch_backproject(p, (T *)p->ybar, ...) then reads it
 template <typename T> ctr_status launch_orbit_bar(const ctr_plan *p, const T *g, cudaStream_t s);
 void bp_tiles(int n, int &tx, int &ty);

@@ -146,12 +146,13 @@ __device__ __forceinline__ void persist_stage_block(int stg, const SliceDesc *__
         return;
     }
     case BS_FWD_SYM: {
-        if (tid >= ORBIT_THREADS) return;
+        if (tid >= OFW_THREADS) return;
         const int s = find_slice(pre, ns, vb);
         const SliceDesc &d = sd[s];
         const int local = vb - pre[s];
-        forward_orbit_body<float, true>(d.ubar, d.n, d.n_jobs, d.M, d.jobs, d.fwe, local % d.fwd_chunks,
-                                        local / d.fwd_chunks);
+        if (d.pair_jobs)
+            ofw_body<2, OFW_JOBS, OFW_SEGS, true>(ofw_args(d), d.fwe, local % d.fwd_chunks, local / d.fwd_chunks);
+        else ofw_body<4, OFW_JOBS, OFW_SEGS, true>(ofw_args(d), d.fwe, local % d.fwd_chunks, local / d.fwd_chunks);
         return;
     }
     default:
@@ -163,7 +164,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
 k_batch_iteration(const SliceDesc *__restrict__ sd, const int *__restrict__ prefix, int ns, GridBarrier *gb,
                   unsigned long long spin_limit)
 {
-    static_assert(32 * BP_TY <= PERSIST_THREADS && FWD_THREADS <= PERSIST_THREADS && ORBIT_THREADS <= PERSIST_THREADS &&
+    static_assert(32 * BP_TY <= PERSIST_THREADS && FWD_THREADS <= PERSIST_THREADS && OFW_THREADS <= PERSIST_THREADS &&
                       OBP_THREADS <= PERSIST_THREADS && FFT_THREADS == PERSIST_THREADS,
                   "stage bodies must fit the persistent CTA");
     constexpr int PHASES = 6;

@@ -1,11 +1,15 @@
 // Kernels of the projectors' symmetric path (OrbitJob): included by radon.cu, inside its
 // unnamed namespace.
 //
-// The sinogram operand of the backprojection lives in *orbit layout*: row j holds, for every
-// detector bin, the NC live channels of job j side by side, zero-padded on both sides far
-// enough that every tile's window of bins lies inside the row.  NC = 4 for plans whose jobs
-// hold up to four angles, 2 for plans of pair jobs (odd view counts; the jobs of channels
-// {0, 1} first, then those of {2, 3}).
+// Both operands are kept in planes of two channels (float2): channels {0, 1} and {2, 3} of a job.
+// On GB300 an 8-byte shared-memory or L1 load of a warp's 32 distinct records takes 2 cycles of
+// an SM, a 16-byte one takes 8 (measured; 64 bytes per cycle instead of 128), so two planes cost
+// half of what one array of float4 does.  NC = 4: plans whose jobs hold up to four angles, both
+// planes read together.  NC = 2: pair plans (odd view counts), each job has one plane; the jobs of
+// channels {0, 1} come first, then those of {2, 3}.
+//
+// The sinogram operand of the backprojection lives in *orbit layout*: NC / 2 rows per job, bin by
+// bin, zero-padded on both sides far enough that every tile's window of bins lies inside the row.
 
 // NC channel values and their packed arithmetic.
 template <int NC> struct Vec;
@@ -17,12 +21,12 @@ template <> struct Vec<2> {
 };
 __device__ __forceinline__ Vec<4> vzero(Vec<4> *) { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
 __device__ __forceinline__ Vec<2> vzero(Vec<2> *) { return {make_float2(0.f, 0.f)}; }
-__device__ __forceinline__ Vec<4> vload(const Vec<4> *p)
+// the record at p in the first plane, `plane` records further in the second
+template <int NC> __device__ __forceinline__ Vec<NC> vload(const float2 *p, int plane)
 {
-    const float4 v = *reinterpret_cast<const float4 *>(p);
-    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+    if constexpr (NC == 4) return {p[0], p[plane]};
+    else return {p[0]};
 }
-__device__ __forceinline__ Vec<2> vload(const Vec<2> *p) { return {*reinterpret_cast<const float2 *>(p)}; }
 __device__ __forceinline__ Vec<4> vadd(Vec<4> x, Vec<4> y) { return {fadd2(x.a, y.a), fadd2(x.b, y.b)}; }
 __device__ __forceinline__ Vec<2> vadd(Vec<2> x, Vec<2> y) { return {fadd2(x.a, y.a)}; }
 __device__ __forceinline__ Vec<4> vsub(Vec<4> x, Vec<4> y) { return {fsub2(x.a, y.a), fsub2(x.b, y.b)}; }
@@ -37,6 +41,8 @@ __device__ __forceinline__ Vec<2> vfma(float w, Vec<2> x, Vec<2> y)
 {
     return {ffma2(make_float2(w, w), x.a, y.a)};
 }
+__device__ __forceinline__ float2 vplane(const Vec<4> &v, int h) { return h == 0 ? v.a : v.b; }
+__device__ __forceinline__ float2 vplane(const Vec<2> &v, int) { return v.a; }
 __device__ __forceinline__ float vget(const Vec<4> &v, int c) { return c == 0 ? v.a.x : c == 1 ? v.a.y : c == 2 ? v.b.x : v.b.y; }
 __device__ __forceinline__ float vget(const Vec<2> &v, int c) { return c == 0 ? v.a.x : v.a.y; }
 
@@ -61,20 +67,14 @@ k_orbit_sino(const S *__restrict__ g, int M, int n_jobs, int list1, int pitch, i
     const int j = blockIdx.y;
     if (k >= M) return;
     const int4 ls = *reinterpret_cast<const int4 *>(jobs[j].l);
-    const size_t o = (size_t)j * pitch + pad + k;
-    if constexpr (NC == 4) {
-        float4 v;
-        v.x = ls.x >= 0 ? ldv(g + (size_t)ls.x * M + k) : 0.f;
-        v.y = ls.y >= 0 ? ldv(g + (size_t)ls.y * M + k) : 0.f;
-        v.z = ls.z >= 0 ? ldv(g + (size_t)ls.z * M + k) : 0.f;
-        v.w = ls.w >= 0 ? ldv(g + (size_t)ls.w * M + k) : 0.f;
-        reinterpret_cast<float4 *>(bar)[o] = v;
-    } else {
-        const int la = j < list1 ? ls.x : ls.z, lb = j < list1 ? ls.y : ls.w;
-        float2 v;
-        v.x = la >= 0 ? ldv(g + (size_t)la * M + k) : 0.f;
-        v.y = lb >= 0 ? ldv(g + (size_t)lb * M + k) : 0.f;
-        reinterpret_cast<float2 *>(bar)[o] = v;
+    const int half = NC == 4 || j < list1 ? 0 : 2;
+    const int l[4] = {ls.x, ls.y, ls.z, ls.w};
+    float2 *row = reinterpret_cast<float2 *>(bar) + (size_t)j * (NC / 2) * pitch + pad + k;
+#pragma unroll
+    for (int h = 0; h < NC / 2; ++h) {
+        const int la = half ? l[2] : l[2 * h], lb = half ? l[3] : l[2 * h + 1];
+        row[(size_t)h * pitch] = make_float2(la >= 0 ? ldv(g + (size_t)la * M + k) : 0.f,
+                                             lb >= 0 ? ldv(g + (size_t)lb * M + k) : 0.f);
     }
 }
 
@@ -91,9 +91,11 @@ k_orbit_sino(const S *__restrict__ g, int M, int n_jobs, int list1, int pitch, i
 // terms are linear in o, so their sums over the jobs are kept once per block (A, and L0, L3
 // for two of the offsets); a pixel adds only its knot, and half of the pixels meet only the
 // right knot, half only the left.  Per block, job and channel that is 12 fused multiply-adds
-// and 5 differences for 8 pixels, and 4 shared-memory bins instead of 16, where an
-// interpolation per pixel takes 24 operations: the shared-memory pipe bounded that form
-// (l1tex 88 %, 8 wavefronts per pixel and warp), the FP32 pipe bounds this one.
+// and 5 differences for 8 pixels, and 4 shared-memory bins, where an interpolation per pixel
+// takes 24 operations and 16 bins.  One R_h^* call, 500^2 / 725 views (pair jobs): 85.6 us with an
+// interpolation per pixel, 38.9 us; 2048^2 / 2048 views: 2280 us, 975 us
+// (the packed FP32 pipe bounds it: fma.f32x2 on three distinct register pairs issues every third
+// cycle, about 130 of the 141 cycles a warp and job take on a scheduler).
 //
 // offsets e0 = (C + 3S)/2, e1 = (C + S)/2, e2 = (C - S)/2, e3 = (C - 3S)/2: pixel (1, 3 - k)
 // sits at +e_k and pixel (0, k) at -e_k.  Jobs with 3 S <= C ("flat") have 0 <= e_k < 1:
@@ -101,21 +103,21 @@ k_orbit_sino(const S *__restrict__ g, int M, int n_jobs, int list1, int pitch, i
 // to 1.42 (two more knots, bins b - 2 .. b + 3).  The jobs of a list are sorted by S / C, so
 // each chunk is a run of flat jobs and a run of steep ones.
 //
-// Bank conflicts: a 16-byte load is served eight lanes at a time; eight lanes hold 4 x 2
-// blocks, whose bins span 6 C + 4 S <= 7.2 plus one: distinct or equal modulo eight.
+// Bank conflicts: an 8-byte load is served sixteen lanes at a time; they hold 8 x 2 blocks,
+// whose bins span 14 C + 4 S <= 14.6 plus one: distinct or equal modulo sixteen.
 // ---------------------------------------------------------------------------
 constexpr int OBP_THREADS = 128;
 constexpr int OBP_JCH = 16;    // jobs per staged chunk (two buffers)
 constexpr int OBP_TJ = 128;    // jobs per table block (one per thread)
 
-template <int NC> constexpr int obp_align() { return 4 / NC; }   // bins per 16 bytes
+constexpr int OBP_WIN = 52;    // bins per staged row (obp_window's most: floor(30 C + 28 S) <= 41, + 9)
 
 // One CTA's inputs (also built from a SliceDesc by the batched stage).
 struct ObpArgs {
     const float *bar;       // sinogram in orbit layout
     const OrbitJob *jobs;
     float *part;            // partial planes [group][v][row][col]
-    int n, pitch, pad, win; // row pitch and left pad in bins; staged bins per job
+    int n, pitch, pad, win; // row pitch and left pad in bins; staged bins per row
     int groups;
     int list[3];            // first job of each list, and the end (NC = 4: one list)
 };
@@ -128,7 +130,7 @@ struct ObpTables {
 };
 
 template <int NC, bool STEEP>
-__device__ __forceinline__ void obp_job(const Vec<NC> *__restrict__ row, uint4 tp, float4 e, int it, int jt,
+__device__ __forceinline__ void obp_job(const float2 *__restrict__ row, uint4 tp, float4 e, int it, int jt,
                                         Vec<NC> &A, Vec<NC> &L0, Vec<NC> &L3, Vec<NC> (&KR)[4], Vec<NC> (&KL)[4])
 {
     using V = Vec<NC>;
@@ -137,8 +139,9 @@ __device__ __forceinline__ void obp_job(const Vec<NC> *__restrict__ row, uint4 t
     const int b = (int)(P >> 31);
     const float f = (float)((unsigned)P & 0x7FFFFFFFu) * 4.656612873077393e-10f;   // 2^-31
     const float fm = f - 1.f;
-    const V *q = row + b;
-    const V g0 = vload(q), g1 = vload(q + 1), gm = vload(q - 1), g2 = vload(q + 2);
+    const float2 *q = row + b;
+    const V g0 = vload<NC>(q, OBP_WIN), g1 = vload<NC>(q + 1, OBP_WIN);
+    const V gm = vload<NC>(q - 1, OBP_WIN), g2 = vload<NC>(q + 2, OBP_WIN);
     const V d0 = vsub(g1, g0), d1 = vsub(g2, g1), dm = vsub(g0, gm);
     const V dr = vsub(d1, d0), dl = vsub(d0, dm);
     A = vadd(A, vfma(f, d0, g0));
@@ -154,7 +157,7 @@ __device__ __forceinline__ void obp_job(const Vec<NC> *__restrict__ row, uint4 t
         KR[3] = vfma(__saturatef(fm + e.w), dr, KR[3]);
         KL[3] = vfma(__saturatef(e.w - f), dl, KL[3]);
     } else {
-        const V g3 = vload(q + 3), gn = vload(q - 2);
+        const V g3 = vload<NC>(q + 3, OBP_WIN), gn = vload<NC>(q - 2, OBP_WIN);
         const V dr2 = vsub(vsub(g3, g2), d1), dl2 = vsub(dm, vsub(gm, gn));
         const float wr = fm + e.x, wl = e.x - f;
         KR[0] = vfma(fmaxf(wr, 0.f), dr, KR[0]);
@@ -170,19 +173,19 @@ template <int NC, bool NAMED>
 __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int bz)
 {
     using V = Vec<NC>;
-    constexpr int AL = obp_align<NC>();
+    constexpr int JROW = NC / 2 * OBP_WIN;                                 // staged records per job
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V *buf = reinterpret_cast<V *>(smem_raw);                              // [2][OBP_JCH][win]
+    float2 *buf = reinterpret_cast<float2 *>(smem_raw);                    // [2][OBP_JCH][NC / 2][OBP_WIN]
     ObpTables tb;
-    tb.pos = reinterpret_cast<uint4 *>(buf + 2 * OBP_JCH * a.win);
+    tb.pos = reinterpret_cast<uint4 *>(buf + 2 * OBP_JCH * JROW);
     tb.e = reinterpret_cast<float4 *>(tb.pos + OBP_TJ);
     tb.row = reinterpret_cast<long long *>(tb.e + OBP_TJ);
     tb.flat = reinterpret_cast<int *>(tb.row + OBP_TJ);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int i0 = by * 32, j0 = bx * 32;
-    // warp: 16 x 16 pixels; eight lanes: 8 x 8 pixels
-    const int it = (warp & 1) * 16 + ((lane >> 3) & 1) * 8 + (lane & 3) * 2;
-    const int jt = (warp >> 1) * 16 + (lane >> 4) * 8 + ((lane >> 2) & 1) * 4;
+    // warp: 16 x 16 pixels; sixteen lanes: 16 x 8 pixels
+    const int it = (warp & 1) * 16 + (lane & 7) * 2;
+    const int jt = (warp >> 1) * 16 + (lane >> 3) * 4;
     const size_t nn = (size_t)a.n * a.n;
     float *pg = a.part + (size_t)bz * 4 * nn;
 #pragma unroll 1
@@ -203,14 +206,14 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
                 const AngleMarch am = a.jobs[t0 + tid].am;                 // canonical P(i, j) = i A + j B + Op
                 const long long C = am.A, S = am.B;
                 const long long P = (long long)i0 * C + (long long)j0 * S + am.Op + ((C + 3 * S) >> 1);
-                const int first = (int)((P >> 32) - 2 + a.pad) & ~(AL - 1);
+                const int first = (int)((P >> 32) - 2 + a.pad) & ~1;                // 16-byte aligned
                 const unsigned long long base = (unsigned long long)(P - ((long long)(first - a.pad) << 32)) >> 1;
                 tb.pos[tid] = make_uint4((unsigned)base, (unsigned)(base >> 32), (unsigned)(C >> 1), (unsigned)(S >> 1));
                 const float c = (float)C * 2.3283064365386963e-10f, s = (float)S * 2.3283064365386963e-10f;   // 2^-32
                 const bool flat = 3 * S <= C;
                 // (e3 = 0 up to rounding either way: both forms of the job then agree)
                 tb.e[tid] = make_float4(0.5f * c + 1.5f * s, 0.5f * c + 0.5f * s, 0.5f * c - 0.5f * s, 0.5f * c - 1.5f * s);
-                tb.row[tid] = (long long)(t0 + tid) * a.pitch + first;
+                tb.row[tid] = (long long)(t0 + tid) * (NC / 2) * a.pitch + first;
                 if (tid == 0 && !flat) *tb.flat = 0;
                 if (flat) {                                                // sorted by S / C: the last flat job
                     bool next = false;
@@ -224,15 +227,16 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
             body_sync<NAMED>();
             const int flat = *tb.flat;
             const int nch = (nt + OBP_JCH - 1) / OBP_JCH;
-            const int units = a.win / AL;                                  // 16-byte units per job
-            auto prefetch = [&](int ch) {
+            const float2 *bar = reinterpret_cast<const float2 *>(a.bar) + 2 * lane;
+            auto prefetch = [&](int ch) {                                  // 16 bytes per lane: win <= 64
                 const int a0 = ch * OBP_JCH, na = min(OBP_JCH, nt - a0);
-                V *dst = buf + (size_t)(ch & 1) * OBP_JCH * a.win;
-                for (int t = warp; t < na; t += OBP_THREADS / 32) {
-                    const float *src = a.bar + (size_t)tb.row[a0 + t] * NC;
-                    float *d = reinterpret_cast<float *>(dst + t * a.win);
-                    for (int w = lane; w < units; w += 32) cp_async16(d + 4 * w, src + 4 * w);
-                }
+                float2 *dst = buf + (ch & 1) * (OBP_JCH * JROW) + 2 * lane;
+                if (2 * lane < a.win)
+                    for (int t = warp; t < na; t += OBP_THREADS / 32) {
+                        const float2 *src = bar + tb.row[a0 + t];
+                        cp_async16(dst + t * JROW, src);
+                        if constexpr (NC == 4) cp_async16(dst + t * JROW + OBP_WIN, src + a.pitch);
+                    }
             };
             prefetch(0);
             cp_async_commit();
@@ -243,14 +247,14 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
                 cp_async_wait<1>();                                        // this thread's copies of chunk ch
                 body_sync<NAMED>();                                        // everyone's
                 const int a0 = ch * OBP_JCH, na = min(OBP_JCH, nt - a0);
-                const V *rows = buf + (size_t)(ch & 1) * OBP_JCH * a.win;
+                const float2 *rows = buf + (ch & 1) * (OBP_JCH * JROW);
                 const int nf = min(max(flat - a0, 0), na);
 #pragma unroll 2
                 for (int t = 0; t < nf; ++t)
-                    obp_job<NC, false>(rows + t * a.win, tb.pos[a0 + t], tb.e[a0 + t], it, jt, A, L0, L3, KR, KL);
+                    obp_job<NC, false>(rows + t * JROW, tb.pos[a0 + t], tb.e[a0 + t], it, jt, A, L0, L3, KR, KL);
 #pragma unroll 2
                 for (int t = nf; t < na; ++t)
-                    obp_job<NC, true>(rows + t * a.win, tb.pos[a0 + t], tb.e[a0 + t], it, jt, A, L0, L3, KR, KL);
+                    obp_job<NC, true>(rows + t * JROW, tb.pos[a0 + t], tb.e[a0 + t], it, jt, A, L0, L3, KR, KL);
                 body_sync<NAMED>();                                        // buffer ch & 1 is refilled next
             }
             cp_async_wait<0>();
@@ -302,16 +306,16 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
 }
 
 template <int NC>
-__global__ void __launch_bounds__(OBP_THREADS, 4) k_backproject_orbit(ObpArgs a)
+__global__ void __launch_bounds__(OBP_THREADS, 5) k_backproject_orbit(ObpArgs a)
 {
     pdl_wait();
     pdl_trigger();
     obp_body<NC, false>(a, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-size_t obp_smem(int win, int nc)
+size_t obp_smem(int nc)
 {
-    return (size_t)2 * OBP_JCH * win * nc * sizeof(float) + OBP_TJ * (sizeof(uint4) + sizeof(float4) + sizeof(long long)) + 16;
+    return (size_t)2 * OBP_JCH * OBP_WIN * nc * sizeof(float) + OBP_TJ * (sizeof(uint4) + sizeof(float4) + sizeof(long long)) + 16;
 }
 
 // the plan's launch arguments
@@ -328,4 +332,254 @@ ObpArgs obp_args(const ctr_plan *p, const float *bar)
     a.groups = p->obp_groups;
     for (int k = 0; k < 3; ++k) a.list[k] = p->job_list[k];
     return a;
+}
+
+// ---------------------------------------------------------------------------
+// Symmetric forward projector.  A warp follows one job's rays down the image rows: lane l
+// carries the pixels q0(m) + l and q0(m) + l + 32, where q0(m) is the first pixel of row m
+// whose coordinate is at least K0 = kb - 1 (the bin before the CTA's first).  P(q0(m), m) - K0
+// = x(m) lies in [0, A) on every row, so pixel slot s (0 <= s < 64) stays within one step
+// A <= 1 of s A + K0 and meets three bins only: its centre c = ceil(s A) and the two beside
+// it.  With z = x + s A - c in (-1, 1) a pixel adds max(z, 0) u to bin c + 1, max(-z, 0) u to
+// bin c - 1 and the rest to bin c; the lane sums u, x u and max(z, 0) u, which give all three.
+// Each pixel of a row is read once by one lane, and x(m) is the same for the whole warp: per
+// slot 3 multiply-adds per channel and one for the weight, per row one conversion.
+// (Marching one bin per lane instead reads two pixels per row, half of the second ones for
+// nothing, and does 4 multiply-adds.)
+//
+// Every job reads the whole orbit image (760 MB in all at 512^2 and 720 views): a CTA takes
+// JOBS adjacent jobs, whose rays nearly coincide, so that they share its lines in L1, and SEGS
+// warps per job that split its rows.  The image rows carry zeros on both sides, so no load is
+// tested.  A chunk of bins is as wide as the slots cover, [kb, kb + nb), nb = floor(64 A) - 1;
+// at the end the slots' three sums are gathered per bin through shared memory, in a fixed order,
+// and all of a job's warps share the epilogue.  One R_h call, 512^2 / 720 views: 69.9 us with the
+// march per bin, 57.2 us; 2048^2 / 2048 views: 2240 us, 1530 us.  The L1 pipe bounds it: an 8-byte
+// load of 32 pixels at an unaligned offset takes 3 wavefronts, 12 a row and warp (48 of the 51
+// cycles that 256 samples of four angles take on an SM at 2048^2).  Tried and slower: float4
+// records (64 cycles), the rows staged in shared memory by cp.async (62: the copies cost as much as
+// the loads), 32 warps a SM at 64 registers, an L1 prefetch 12 to 32 rows ahead (no change).
+// ---------------------------------------------------------------------------
+constexpr int OFW_JOBS = 2, OFW_SEGS = 2, OFW_THREADS = 32 * OFW_JOBS * OFW_SEGS;   // of the batched stage
+
+struct OfwArgs {
+    const float *ubar;      // orbit image
+    const OrbitJob *jobs;
+    int n, M, n_jobs, list1;
+};
+
+template <int NC, int JOBS, int SEGS, bool NAMED>
+__device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<float> &epi, int bx, int by)
+{
+    using V = Vec<NC>;
+    constexpr int STRIPS = OFW_LANES / 32, LN = OFW_LANES;
+    constexpr int H = NC / 2, NT = 32 * SEGS;
+    __shared__ float2 s_part[JOBS][SEGS][H][3 * LN];   // per plane: the slots' sums for bins c, c + 1, c - 1
+    __shared__ int s_first[JOBS][LN + 4];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int slot = warp % JOBS, seg = warp / JOBS;
+    // the CTA's jobs: groups of JOBS within each list
+    const int g0 = (a.list1 + JOBS - 1) / JOBS;
+    const int j0 = by < g0 ? by * JOBS : a.list1 + (by - g0) * JOBS;
+    const int nj = min(JOBS, (by < g0 ? a.list1 : a.n_jobs) - j0), jb = j0 + slot;
+    const int half = NC == 4 || by < g0 ? 0 : 2;      // (pair plans: the list's channels)
+    // chunk width: the narrowest of the CTA's jobs, so that their bins coincide
+    long long amin = 1ll << 32;
+#pragma unroll
+    for (int q = 0; q < JOBS; ++q)
+        if (q < nj) amin = min(amin, a.jobs[j0 + q].am.A);
+    const int nb = (int)((LN * amin) >> 32) - 1;
+    const int kb = bx * nb;
+    if (kb >= a.M) return;                            // CTA-uniform
+    const bool active = slot < nj;                    // warp-uniform
+    V S[STRIPS], X[STRIPS], Pp[STRIPS], Nn[STRIPS];   // sums of u, x u, max(z, 0) u; of max(-z, 0) u at the end
+#pragma unroll
+    for (int t = 0; t < STRIPS; ++t) S[t] = X[t] = Nn[t] = Pp[t] = vzero((V *)nullptr);
+    const AngleMarch am = a.jobs[active ? jb : j0].am;
+    const long long A = am.A, B = am.B, K0 = (long long)(kb - 1) << 32;
+    // rows on which a slot may lie in the image, rounded out: q0(m) stays within [-66, n + 3]
+    // there, inside the pads (the estimate is off by far less than a pixel: |Q0| < 2^14 wherever
+    // a row meets the image)
+    const float Q0 = (float)(K0 - am.Op) * (am.kA * 2.3283064365386963e-10f);
+    int mlo, mhi;
+    rows_in<true>(Q0, am.binv, -(float)LN - 1.f, (float)a.n + 1.f, a.n, mlo, mhi);
+    if (SEGS > 1 && mlo <= mhi) {                     // this warp's part of the rows
+        const int per = (mhi - mlo + SEGS) / SEGS;
+        mlo += seg * per;
+        mhi = min(mhi, mlo + per - 1);
+    }
+    if (active && mlo <= mhi) {
+        int q = (int)ceilf(Q0 - (float)mlo * ((float)B / (float)A));
+        long long x = (long long)q * A + (long long)mlo * B + am.Op - K0;
+        while (x < 0) { x += A; ++q; }                // (the estimate is off by one at most)
+        while (x >= A) { x -= A; --q; }
+        // x + B >= A: the next row's first pixel moves left.  The bound A - B is 2^32 only for
+        // A = 2^32, B = 0, where x never moves: bound and x are kept one unit lower there
+        const unsigned bound = (unsigned)min(A - B, 0xFFFFFFFFll);
+        unsigned r = B == 0 ? min((unsigned)x, 0xFFFFFFFEu) : (unsigned)x;
+        const unsigned B32 = (unsigned)B, BA32 = (unsigned)(B - A);
+        float phi[STRIPS];
+#pragma unroll
+        for (int t = 0; t < STRIPS; ++t) {
+            const long long y = (long long)(lane + 32 * t) * A;
+            phi[t] = -(float)(unsigned)(-y) * 2.3283064365386963e-10f;   // y - ceil(y), y in 2^-32 bins
+        }
+        const int pitch = orbit_pitch(a.n), plane = pitch * a.n;
+        const float2 *ub = reinterpret_cast<const float2 *>(a.ubar) + (half ? plane : 0) + ORBIT_PAD + lane;
+        const float2 *ub2 = ub + plane;
+        int off = mlo * pitch + q;
+#pragma unroll 8
+        for (int m = mlo; m <= mhi; ++m) {
+            V v[STRIPS];
+#pragma unroll
+            for (int t = 0; t < STRIPS; ++t) {
+                v[t].a = __ldg(ub + off + 32 * t);
+                if constexpr (NC == 4) v[t].b = __ldg(ub2 + off + 32 * t);
+            }
+            const float xf = (float)r;                // x, in 2^-32 bins
+#pragma unroll
+            for (int t = 0; t < STRIPS; ++t) {
+                S[t] = vadd(S[t], v[t]);
+                X[t] = vfma(xf, v[t], X[t]);
+                Pp[t] = vfma(__saturatef(fmaf(xf, 2.3283064365386963e-10f, phi[t])), v[t], Pp[t]);
+            }
+            const bool step = r >= bound;
+            r += step ? BA32 : B32;
+            off += step ? pitch - 1 : pitch;
+        }
+        // max(-z, 0) = max(z, 0) - z, z = x + phi
+#pragma unroll
+        for (int t = 0; t < STRIPS; ++t)
+            Nn[t] = vfma(-phi[t], S[t], vfma(-2.3283064365386963e-10f, X[t], Pp[t]));
+    }
+#pragma unroll
+    for (int t = 0; t < STRIPS; ++t) {
+        const V mid = vsub(S[t], vadd(Pp[t], Nn[t]));
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            float2 *q = s_part[slot][seg][h] + lane + 32 * t;
+            q[0] = vplane(mid, h);
+            q[LN] = vplane(Pp[t], h);
+            q[2 * LN] = vplane(Nn[t], h);
+        }
+    }
+    // the slots of centre v are first[v] .. first[v + 1] - 1
+    int *first = s_first[slot];
+    if (seg == 0) {
+        for (int e = lane; e < LN + 4; e += 32) first[e] = LN;
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < STRIPS; ++t) {
+            const int q = lane + 32 * t;
+            const int c = (int)((q * A + 0xFFFFFFFFll) >> 32), cp = (int)(((q - 1) * A + 0xFFFFFFFFll) >> 32);
+            if (q == 0 || c > cp) first[c] = q;       // A <= 1: no centre is skipped
+        }
+    }
+    // from here on the job's NT threads share its bins: one bin and plane each
+    const int tj = seg * 32 + lane;
+    constexpr int ITEMS = (LN * H + NT - 1) / NT;
+    const bool pre = epi.mode == 1 || epi.mode == 2;
+    float ops[2][5];                                  // the first item's operands, on their way meanwhile
+    auto fetch = [&](int it) {
+        const int b = it % LN, h = it / LN, k = kb + b;
+        const bool ok = active && it < LN * H && b < nb && k < a.M;
+        const float *src[5] = {epi.v1b, epi.dw, epi.da, epi.dlo, epi.dhi};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int l = ok ? a.jobs[jb].l[half + 2 * h + c] : -1;
+#pragma unroll
+            for (int o = 0; o < 5; ++o) ops[c][o] = l >= 0 ? src[o][(size_t)l * a.M + k] : 0.f;
+        }
+    };
+    if (pre) fetch(tj);
+    body_sync<NAMED>();
+    if constexpr (SEGS > 1) {
+        for (int e = tj; e < 3 * LN * H; e += NT) {
+            const int h = e / (3 * LN), q = e - h * (3 * LN);
+            float2 v = s_part[slot][0][h][q];
+#pragma unroll
+            for (int z = 1; z < SEGS; ++z) v = fadd2(v, s_part[slot][z][h][q]);
+            s_part[slot][0][h][q] = v;
+        }
+        body_sync<NAMED>();
+    }
+    if (!active) return;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int it = tj + i * NT, b = it % LN, h = it / LN, k = kb + b;
+        if (i > 0 && pre) fetch(it);
+        if (it >= LN * H || b >= nb || k >= a.M) continue;
+        // bin kb + b is centre c = b + 1
+        const float2 *acc = s_part[slot][0][h];
+        float2 g = make_float2(0.f, 0.f);
+        const int q0 = first[b], q1 = first[b + 1], q2 = first[b + 2], q3 = first[b + 3];
+        for (int q = q0; q < q1; ++q) g = fadd2(g, acc[LN + q]);
+        for (int q = q1; q < q2; ++q) g = fadd2(g, acc[q]);
+        for (int q = q2; q < q3; ++q) g = fadd2(g, acc[2 * LN + q]);
+        float y[2] = {0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            const int l = a.jobs[jb].l[half + 2 * h + c];
+            if (l < 0) continue;
+            float *yd = epi.ybar ? &y[c] : nullptr;
+            const float val = c == 0 ? g.x : g.y;
+            if (pre)
+                forward_epilogue_pre(epi, (size_t)l * a.M + k, val, ops[c][0], ops[c][1], ops[c][2], ops[c][3], ops[c][4], yd);
+            else forward_epilogue(epi, (size_t)l * a.M + k, val, yd);
+        }
+        if (epi.ybar)
+            reinterpret_cast<float2 *>(epi.ybar)[((size_t)jb * H + h) * epi.ypitch + epi.ypad + k] = make_float2(y[0], y[1]);
+    }
+}
+
+template <int NC, int JOBS, int SEGS>
+__global__ void __launch_bounds__(32 * JOBS * SEGS, 24 / (JOBS * SEGS))
+k_forward_orbit(OfwArgs a, ForwardEpi<float> epi)
+{
+    pdl_wait();
+    pdl_trigger();
+    // chunks from the detector's middle outwards: the long rays first, the short ones fill the tail
+    const int c = blockIdx.y, mid = (gridDim.y - 1) / 2;
+    ofw_body<NC, JOBS, SEGS, false>(a, epi, c & 1 ? mid + (c + 1) / 2 : mid - c / 2, blockIdx.x);
+}
+
+// CTA rows of the job lists in groups of `jobs`
+int ofw_groups(const ctr_plan *p, int jobs)
+{
+    return (p->job_list[1] + jobs - 1) / jobs + (p->n_jobs - p->job_list[1] + jobs - 1) / jobs;
+}
+
+template <int JOBS, int SEGS>
+void launch_forward_orbit_shape(const ctr_plan *p, const float *ub, const ForwardEpi<float> &epi, cudaStream_t s)
+{
+    const dim3 grid(ofw_groups(p, JOBS), p->fwd_chunks);
+    launch_pdl(p->pdl != 0, p->pair_jobs ? k_forward_orbit<2, JOBS, SEGS> : k_forward_orbit<4, JOBS, SEGS>, grid,
+               dim3(32 * JOBS * SEGS), 0, s, OfwArgs{ub, p->d_jobs, p->n, p->M, p->n_jobs, p->job_list[1]}, epi);
+}
+
+// The launch shape (jobs * 16 + segments): the one ctr_plan_set_fwd_shape chose, or for its default
+// (1, 4) the one measured best for the number of (job, chunk) pairs there are: with many, two
+// adjacent jobs share their image lines in L1 (four-channel jobs 2048^2: (2, 4) 1530 us, (1, 4)
+// 1740; 512^2 with 3077 pairs: 57 either way.  Pair jobs 2048^2 / 2047 views: (2, 2) 1813, (1, 4) 1879;
+// 500^2 / 725 with 6171 pairs: 61.6 and 62.4); with few, splitting rows over four warps matters more
+// (256^2: (1, 4) 17.8, (2, 2) 24.1).
+int ofw_shape(const ctr_plan *p)
+{
+    const int shape = p->fwd_slots * 16 + p->fwd_segs;
+    if (shape != 1 * 16 + 4) return shape;
+    const long long pairs = (long long)p->n_jobs * p->fwd_chunks;
+    if (p->pair_jobs) return pairs >= 8000 ? 2 * 16 + 2 : shape;
+    return pairs >= 4000 ? 2 * 16 + 4 : shape;
+}
+
+void launch_forward_orbit(const ctr_plan *p, const float *ub, const ForwardEpi<float> &epi, cudaStream_t s)
+{
+    switch (ofw_shape(p)) {
+    case 1 * 16 + 2: launch_forward_orbit_shape<1, 2>(p, ub, epi, s); break;
+    case 1 * 16 + 8: launch_forward_orbit_shape<1, 8>(p, ub, epi, s); break;
+    case 2 * 16 + 2: launch_forward_orbit_shape<2, 2>(p, ub, epi, s); break;
+    case 2 * 16 + 4: launch_forward_orbit_shape<2, 4>(p, ub, epi, s); break;
+    case 4 * 16 + 2: launch_forward_orbit_shape<4, 2>(p, ub, epi, s); break;
+    case 4 * 16 + 1: launch_forward_orbit_shape<4, 1>(p, ub, epi, s); break;
+    default: launch_forward_orbit_shape<1, 4>(p, ub, epi, s); break;
+    }
 }

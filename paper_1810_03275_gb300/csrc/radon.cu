@@ -18,7 +18,8 @@
 //    every lane of a warp stays inside the image run without bounds checks.
 //    No atomics; each output bin is written once.
 // Both kernels derive each weight from the same integer P (see ctr_internal.cuh),
-// so they are transposes of one matrix, bit for bit in the weights.
+// so they are transposes of one matrix.  Plans whose angles are symmetric images of
+// one another take the kernels of orbit.cuh instead, which use the same integers.
 #include <algorithm>
 #include <type_traits>
 
@@ -73,10 +74,6 @@ __device__ __forceinline__ int bin_of(long long P, int F)
 #define CTR_FWD_UNROLL 8
 #endif
 constexpr int FWD_UNROLL = CTR_FWD_UNROLL;   // rows per unrolled step of the ray march
-#ifndef CTR_FWD_UNROLL_ORBIT
-#define CTR_FWD_UNROLL_ORBIT 8
-#endif
-constexpr int FWD_UNROLL_ORBIT = CTR_FWD_UNROLL_ORBIT;
 
 // x / d for x, d >= 0 with x d < 2^32 as the high word of x m, m = floor((2^32 - 1) / d) + 1
 // (then m - 2^32 / d < 1 and the error x (m - 2^32/d) / 2^32 stays below 1/d, so the floor is
@@ -556,57 +553,51 @@ k_forward(const S *__restrict__ u, const S *__restrict__ uT, int n, int N, int M
 // job's up to four angles, reading the four channels of the orbit image at once.
 // ---------------------------------------------------------------------------
 
-// Orbit-image records: the four channels of one pixel, FP32 (float4) or bfloat16
-// (uint2, channel 0 in the low half of x).  rec_f32 widens a record to FP32.
-template <typename S> struct OrbitRec;
-template <> struct OrbitRec<float> { using type = float4; };
-template <> struct OrbitRec<__nv_bfloat16> { using type = uint2; };
-__device__ __forceinline__ float4 rec_f32(float4 v) { return v; }
-__device__ __forceinline__ float4 rec_f32(uint2 v)
+// The orbit image: channel v of the canonical march pixel (q, m) is u(T_v^{-1}(q, m)),
+//     ubar[m][q] = (u[q][m], u[n-1-q][m], u[m][q], u[n-1-m][q]),
+// FP32 (a BF16 plan's operand is widened here).  Rows of
+// orbit_pitch pixels, pixel 0 at ORBIT_PAD; the pads keep the zeros they got when the plan was
+// made.  Two planes (float2): channels {0, 1}, then {2, 3}.
+__device__ __forceinline__ void orbit_store(float *__restrict__ ubar, size_t plane, size_t o, float a, float b, float c,
+                                            float d)
 {
-    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u), __uint_as_float(v.y << 16),
-                       __uint_as_float(v.y & 0xFFFF0000u));
-}
-__device__ __forceinline__ float4 make_rec(float a, float b, float c, float d) { return make_float4(a, b, c, d); }
-__device__ __forceinline__ uint2 make_rec(__nv_bfloat16 a, __nv_bfloat16 b, __nv_bfloat16 c, __nv_bfloat16 d)
-{
-    return make_uint2((unsigned)__bfloat16_as_ushort(a) | ((unsigned)__bfloat16_as_ushort(b) << 16),
-                      (unsigned)__bfloat16_as_ushort(c) | ((unsigned)__bfloat16_as_ushort(d) << 16));
+    reinterpret_cast<float2 *>(ubar)[o] = make_float2(a, b);
+    reinterpret_cast<float2 *>(ubar)[plane + o] = make_float2(c, d);
 }
 
-// ubar[m][q] = (u[q][m], u[n-1-q][m], u[m][q], u[n-1-m][q]): channel v holds
-// u(T_v^{-1}(q, m)) for the canonical march pixel (q, m) (pick q = i, march m = j).
 // 32 x 32 tiles: four coalesced tile loads (two of them transposed through shared
 // memory), one coalesced record store per pixel.
 template <typename S>
-__device__ __forceinline__ void orbit_image_body(const S *__restrict__ u, typename OrbitRec<S>::type *__restrict__ ubar,
-                                                 int n, int bx, int by)
+__device__ __forceinline__ void orbit_image_body(const S *__restrict__ u, float *__restrict__ ubar, int n, int bx, int by)
 {
-    __shared__ S tA[32][33], tB[32][33], tC[32][33], tD[32][33];
+    __shared__ float tA[32][33], tB[32][33], tC[32][33], tD[32][33];
+    const size_t pitch = orbit_pitch(n), plane = pitch * n;
+    ubar += 2 * ORBIT_PAD;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int q0 = bx * 32, m0 = by * 32;
     for (int r = ty; r < 32; r += 8) {
         const int mr = m0 + r, qc = q0 + tx;          // tiles A, B: rows m, columns q
         if (mr < n && qc < n) {
-            tA[r][tx] = u[(size_t)mr * n + qc];
-            tB[r][tx] = u[(size_t)(n - 1 - mr) * n + qc];
+            tA[r][tx] = ldv(u + (size_t)mr * n + qc);
+            tB[r][tx] = ldv(u + (size_t)(n - 1 - mr) * n + qc);
         }
         const int qr = q0 + r, mc = m0 + tx;          // tiles C, D: rows q, columns m
         if (qr < n && mc < n) {
-            tC[r][tx] = u[(size_t)qr * n + mc];
-            tD[r][tx] = u[(size_t)(n - 1 - qr) * n + mc];
+            tC[r][tx] = ldv(u + (size_t)qr * n + mc);
+            tD[r][tx] = ldv(u + (size_t)(n - 1 - qr) * n + mc);
         }
     }
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
         const int m = m0 + r, q = q0 + tx;
-        if (m < n && q < n) ubar[(size_t)m * n + q] = make_rec(tC[tx][r], tD[tx][r], tA[r][tx], tB[r][tx]);
+        if (m < n && q < n)
+            orbit_store(ubar, plane, (size_t)m * pitch + q, tC[tx][r], tD[tx][r], tA[r][tx], tB[r][tx]);
     }
 }
 
 template <typename S>
 __global__ void __launch_bounds__(256)
-k_orbit_image(const S *__restrict__ u, typename OrbitRec<S>::type *__restrict__ ubar, int n)
+k_orbit_image(const S *__restrict__ u, float *__restrict__ ubar, int n)
 {
     pdl_wait();
     pdl_trigger();
@@ -619,11 +610,13 @@ k_orbit_image(const S *__restrict__ u, typename OrbitRec<S>::type *__restrict__ 
 // its forward neighbours comes from tile A (rows m, columns q, plus a one-pixel halo), so
 // the kernel waits on global memory once; the arithmetic is that of tv_dual_at.
 __global__ void __launch_bounds__(256)
-k_orbit_image_tv(const float *__restrict__ u, OrbitRec<float>::type *__restrict__ ubar, int n, TvDualJob<float> tv)
+k_orbit_image_tv(const float *__restrict__ u, float *__restrict__ ubar, int n, TvDualJob<float> tv)
 {
     pdl_wait();
     pdl_trigger();
     __shared__ float tA[33][33], tB[32][33], tC[32][33], tD[32][33];
+    const size_t pitch = orbit_pitch(n), plane = pitch * n;
+    ubar += 2 * ORBIT_PAD;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int q0 = blockIdx.x * 32, m0 = blockIdx.y * 32;
     const size_t nn = (size_t)n * n;
@@ -656,7 +649,8 @@ k_orbit_image_tv(const float *__restrict__ u, OrbitRec<float>::type *__restrict_
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
         const int m = m0 + r, q = q0 + tx;
-        if (m < n && q < n) ubar[(size_t)m * n + q] = make_rec(tC[tx][r], tD[tx][r], tA[r][tx], tB[r][tx]);
+        if (m < n && q < n)
+            orbit_store(ubar, plane, (size_t)m * pitch + q, tC[tx][r], tD[tx][r], tA[r][tx], tB[r][tx]);
     }
     const float st = tv.sigma * tv.tau;
 #pragma unroll
@@ -689,13 +683,7 @@ k_orbit_image_tv(const float *__restrict__ u, OrbitRec<float>::type *__restrict_
     }
 }
 
-// Asynchronous copies global -> shared (cp.async): one 4-byte element (src_size 0 stores
-// zero and reads nothing), commit and wait on this thread's groups.
-__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
+// Asynchronous copies global -> shared (cp.async): commit, and wait on this thread's groups.
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
@@ -743,453 +731,6 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c)
 #else
     return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
 #endif
-}
-
-__device__ __forceinline__ void acc4(float4 &Su, float4 &Sf, float4 v, float f)
-{
-#if CTR_F32X2
-    const float2 f2 = make_float2(f, f);
-    const float2 v01 = make_float2(v.x, v.y), v23 = make_float2(v.z, v.w);
-    const float2 u01 = fadd2(make_float2(Su.x, Su.y), v01), u23 = fadd2(make_float2(Su.z, Su.w), v23);
-    const float2 s01 = ffma2(f2, v01, make_float2(Sf.x, Sf.y)), s23 = ffma2(f2, v23, make_float2(Sf.z, Sf.w));
-    Su = make_float4(u01.x, u01.y, u23.x, u23.y);
-    Sf = make_float4(s01.x, s01.y, s23.x, s23.y);
-    return;
-#endif
-    Su.x += v.x;
-    Su.y += v.y;
-    Su.z += v.z;
-    Su.w += v.w;
-    Sf.x = fmaf(f, v.x, Sf.x);
-    Sf.y = fmaf(f, v.y, Sf.y);
-    Sf.z = fmaf(f, v.z, Sf.z);
-    Sf.w = fmaf(f, v.w, Sf.w);
-}
-
-// What the march reads at a pixel: the whole orbit record (four channels), or for a pair
-// job (whose angles all sit in channels {0, 1} or {2, 3}) the two live channels of the
-// FP32 record as one 8-byte load.  acc_v accumulates each channel exactly as acc4 does.
-template <typename R>
-struct RecLoad {
-    using V = float4;
-    const R *__restrict__ ub;
-    __device__ __forceinline__ float4 operator()(int off) const { return rec_f32(ub[off]); }
-    __device__ __forceinline__ static float4 zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-};
-struct PairLoad {
-    using V = float2;
-    const float2 *__restrict__ ub2;     // (const float2 *)ub + h: channels 2h, 2h + 1 of each record
-    __device__ __forceinline__ float2 operator()(int off) const { return ub2[2 * (size_t)off]; }
-    __device__ __forceinline__ static float2 zero() { return make_float2(0.f, 0.f); }
-};
-__device__ __forceinline__ void acc_v(float4 &Su, float4 &Sf, float4 v, float f) { acc4(Su, Sf, v, f); }
-__device__ __forceinline__ void acc_v(float2 &Su, float2 &Sf, float2 v, float f)
-{
-    Su = fadd2(Su, v);
-    Sf = ffma2(make_float2(f, f), v, Sf);
-}
-
-// The canonical march (flip 0, B >= 0) over `rows` rows of the orbit image; the
-// state and the second-pixel rule are those of march32.
-template <bool BPOS, bool CHECK, typename L>
-__device__ __forceinline__ void march_orbit(const L &ld, int n, int rows, unsigned &r, int &q, int &off,
-                                            unsigned A32, unsigned lim, unsigned B32, unsigned thr,
-                                            typename L::V &Su, typename L::V &Sf)
-{
-    using V = typename L::V;
-#pragma unroll FWD_UNROLL_ORBIT
-    for (int rr = 0; rr < rows; ++rr) {
-        V v1, v2;
-        if constexpr (CHECK) {
-            v1 = ((unsigned)q < (unsigned)n) ? ld(off) : L::zero();
-            v2 = (r < lim && (unsigned)(q + 1) < (unsigned)n) ? ld(off + 1) : L::zero();
-        } else {
-            v1 = ld(off);
-            v2 = r < lim ? ld(off + 1) : L::zero();
-        }
-        acc_v(Su, Sf, v1, one_plus_frac32u(r));
-        acc_v(Su, Sf, v2, one_plus_frac32u(r + A32));
-        if constexpr (BPOS) {
-            const bool s = r >= thr;
-            r += s ? B32 - A32 : B32;
-            off += s ? n - 1 : n;
-            if constexpr (CHECK) q -= s ? 1 : 0;
-        } else {
-            const bool s = r < thr;
-            r += s ? A32 - thr : 0u - thr;
-            off += s ? n + 1 : n;
-            if constexpr (CHECK) q += s ? 1 : 0;
-        }
-    }
-}
-
-template <bool BPOS, typename L>
-__device__ __forceinline__ void march_orbit_rows(const L &ub, int n, long long K, const AngleMarch &am, int mlo,
-                                                 int mhi, int ilo, int ihi, typename L::V &Su, typename L::V &Sf)
-{
-    const long long A = am.A, B = am.B;
-    const long long qa = ceil_div_ll(K - (long long)mlo * B - am.Op, A);
-    unsigned r = (unsigned)(qa * A + (long long)mlo * B + am.Op - K);
-    int q = (int)qa;
-    int off = mlo * n + q;
-    const unsigned A32 = (unsigned)A;
-    const unsigned lim = (unsigned)((1ll << 32) - A);
-    const unsigned B32 = (unsigned)B;
-    const unsigned thr = BPOS ? (unsigned)(A - B) : (unsigned)(-B);
-    if (ilo > ihi) {
-        march_orbit<BPOS, true>(ub, n, mhi - mlo + 1, r, q, off, A32, lim, B32, thr, Su, Sf);
-        return;
-    }
-    march_orbit<BPOS, true>(ub, n, ilo - mlo, r, q, off, A32, lim, B32, thr, Su, Sf);
-    march_orbit<BPOS, false>(ub, n, ihi - ilo + 1, r, q, off, A32, lim, B32, thr, Su, Sf);
-    q = off - (ihi + 1) * n;
-    march_orbit<BPOS, true>(ub, n, mhi - ihi, r, q, off, A32, lim, B32, thr, Su, Sf);
-}
-
-__device__ __forceinline__ void orbit_out(const ForwardEpi<float> &epi, int job, int c, int l, int M, int k, int lane,
-                                          float Su, float Sf, const float *pre = nullptr)
-{
-    const float Bk = Sf - Su, Ak = Su - Bk;
-    const float Bprev = __shfl_up_sync(0xffffffffu, Bk, 1);
-    if (l >= 0 && lane >= 1 && k < M) {
-        float *yd = epi.ybar ? epi.ybar + ((size_t)job * epi.ypitch + epi.ypad + k) * epi.ync + (c & (epi.ync - 1)) : nullptr;
-        if (pre) forward_epilogue_pre(epi, (size_t)l * M + k, Ak + Bprev, pre[0], pre[32], pre[64], pre[96], pre[128], yd);
-        else forward_epilogue(epi, (size_t)l * M + k, Ak + Bprev, yd);
-    }
-}
-
-// The data-dual epilogue's per-bin operands (v1b, w, a, lo, hi) of the lane's four angles,
-// copied into shared memory [angle][operand][lane] at the start of the march so that their
-// latency is hidden behind it (modes 1 and 2 read them; each (angle, bin) belongs to one lane).
-__device__ __forceinline__ void orbit_epi_prefetch(const ForwardEpi<float> &epi, int4 ls, int M, int k, int lane,
-                                                   float *s)
-{
-    const int l4[4] = {ls.x, ls.y, ls.z, ls.w};
-    const float *src[5] = {epi.v1b, epi.dw, epi.da, epi.dlo, epi.dhi};
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const bool ok = l4[c] >= 0 && lane >= 1 && k < M;
-        const size_t r = ok ? (size_t)l4[c] * M + k : 0;
-#pragma unroll
-        for (int o = 0; o < 5; ++o) cp_async4(s + (c * 5 + o) * 32 + lane, src[o] + r, ok);
-    }
-    cp_async_commit();
-}
-
-#ifndef CTR_ORBIT_SEGS
-#define CTR_ORBIT_SEGS 4
-#endif
-constexpr int ORBIT_SEGS = CTR_ORBIT_SEGS;    // row segments of a job's rays (one warp each)
-#ifndef CTR_ORBIT_SLOTS
-#define CTR_ORBIT_SLOTS 1
-#endif
-// adjacent jobs per CTA; 1 (128-thread CTAs, 8 per SM) measured fastest: co-resident CTAs of
-// adjacent jobs share the SM's L1 anyway, and small CTAs retire and refill sooner
-constexpr int ORBIT_SLOTS = CTR_ORBIT_SLOTS;
-constexpr int ORBIT_THREADS = 32 * ORBIT_SLOTS * ORBIT_SEGS;
-#ifndef CTR_ORBIT_MINB
-#define CTR_ORBIT_MINB 8
-#endif
-
-// Warp w of the CTA takes job by*ORBIT_SLOTS + w % ORBIT_SLOTS, bins bx*31 + [0, 31) and
-// the (w / ORBIT_SLOTS)-th of ORBIT_SEGS equal parts of the rows its rays cross; the parts' sums
-// are added in a fixed order through shared memory.
-template <typename S, bool NAMED = false, int SEGS = ORBIT_SEGS, int SLOTS = ORBIT_SLOTS, bool PAIRS = false>
-__device__ __forceinline__ void forward_orbit_body(const typename OrbitRec<S>::type *__restrict__ ubar, int n,
-                                                   int n_jobs, int M, const OrbitJob *__restrict__ jobs,
-                                                   const ForwardEpi<float> &epi, int bx, int by)
-{
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int slot = warp % SLOTS, seg = warp / SLOTS;
-    const int jb = by * SLOTS + slot;
-    const int kb = bx * 31;
-    const int k = kb + lane - 1;
-    const bool active = jb < n_jobs && kb < M;        // warp-uniform
-    float4 Su = make_float4(0.f, 0.f, 0.f, 0.f), Sf = Su;
-    int4 ls = make_int4(-1, -1, -1, -1);             // the job's angles
-    __shared__ float s_epi[SLOTS][4 * 5 * 32];
-    const bool pre = (epi.mode == 1 || epi.mode == 2) && seg == 0 && active;   // warp-uniform
-    if (active) {
-        const AngleMarch am = jobs[jb].am;
-        ls = *reinterpret_cast<const int4 *>(jobs[jb].l);
-        if (pre) orbit_epi_prefetch(epi, ls, M, k, lane, s_epi[slot]);
-        const float Q0 = (float)k * am.kA - am.oA;
-        int mlo, mhi;
-        rows_in<true>(Q0, am.binv, -3.f, (float)n + 1.f, n, mlo, mhi);
-        int mlo_w = __reduce_min_sync(0xffffffffu, mlo);
-        int mhi_w = __reduce_max_sync(0xffffffffu, mhi);
-        if (mlo_w <= mhi_w) {
-            int ilo, ihi;
-            rows_in<false>(Q0, am.binv, 0.5f, (float)n - 3.5f, n, ilo, ihi);
-            int ilo_w = max(__reduce_max_sync(0xffffffffu, ilo), mlo_w);
-            int ihi_w = min(__reduce_min_sync(0xffffffffu, ihi), mhi_w);
-            if (SEGS > 1) {                     // this warp's part of the rows
-                const int per = (mhi_w - mlo_w + SEGS) / SEGS;
-                const int a = mlo_w + seg * per, b = min(mhi_w, a + per - 1);
-                mlo_w = a;
-                mhi_w = b;
-                ilo_w = max(ilo_w, a);
-                ihi_w = min(ihi_w, b);
-            }
-            if (mlo_w <= mhi_w) {
-                const long long K = (long long)k << 32;
-                // a pair job (channels {0, 1} or {2, 3} only; odd view counts give only these)
-                // reads and accumulates its two live channels; the others stay zero as they
-                // would in the four-channel march
-                bool done = false;
-                if constexpr (PAIRS && std::is_same<S, float>::value) {
-                    const int pair = (ls.z < 0 && ls.w < 0) ? 1 : ((ls.x < 0 && ls.y < 0) ? 2 : 0);
-                    if (pair) {
-                        const PairLoad ld{reinterpret_cast<const float2 *>(ubar) + (pair - 1)};
-                        float2 su = make_float2(0.f, 0.f), sf = su;
-                        if (am.B > 0) march_orbit_rows<true>(ld, n, K, am, mlo_w, mhi_w, ilo_w, ihi_w, su, sf);
-                        else march_orbit_rows<false>(ld, n, K, am, mlo_w, mhi_w, ilo_w, ihi_w, su, sf);
-                        if (pair == 1) {
-                            Su.x = su.x; Su.y = su.y; Sf.x = sf.x; Sf.y = sf.y;
-                        } else {
-                            Su.z = su.x; Su.w = su.y; Sf.z = sf.x; Sf.w = sf.y;
-                        }
-                        done = true;
-                    }
-                }
-                if (!done) {
-                    const RecLoad<typename OrbitRec<S>::type> ld{ubar};
-                    if (am.B > 0) march_orbit_rows<true>(ld, n, K, am, mlo_w, mhi_w, ilo_w, ihi_w, Su, Sf);
-                    else march_orbit_rows<false>(ld, n, K, am, mlo_w, mhi_w, ilo_w, ihi_w, Su, Sf);
-                }
-            }
-        }
-    }
-    if constexpr (SEGS > 1) {
-        __shared__ float4 s_part[SEGS > 1 ? SEGS - 1 : 1][2][SLOTS][32];
-        if (seg > 0) {
-            s_part[seg - 1][0][slot][lane] = Su;
-            s_part[seg - 1][1][slot][lane] = Sf;
-        }
-        body_sync<NAMED>();
-        if (seg > 0) return;
-#pragma unroll
-        for (int z = 0; z < SEGS - 1; ++z) {
-            const float4 a = s_part[z][0][slot][lane], b = s_part[z][1][slot][lane];
-            Su.x += a.x; Su.y += a.y; Su.z += a.z; Su.w += a.w;
-            Sf.x += b.x; Sf.y += b.y; Sf.z += b.z; Sf.w += b.w;
-        }
-    }
-    if (!active) return;
-    if (pre) cp_async_wait<0>();                      // this lane's own copies: no barrier needed
-    const float *pe = pre ? s_epi[slot] + lane : nullptr;
-    orbit_out(epi, jb, 0, ls.x, M, k, lane, Su.x, Sf.x, pe ? pe + 0 * 160 : nullptr);
-    orbit_out(epi, jb, 1, ls.y, M, k, lane, Su.y, Sf.y, pe ? pe + 1 * 160 : nullptr);
-    orbit_out(epi, jb, 2, ls.z, M, k, lane, Su.z, Sf.z, pe ? pe + 2 * 160 : nullptr);
-    orbit_out(epi, jb, 3, ls.w, M, k, lane, Su.w, Sf.w, pe ? pe + 3 * 160 : nullptr);
-}
-
-// SLOTS adjacent jobs per CTA (their rays nearly coincide, so they share the orbit
-// image's lines in L1) and SEGS warps per job splitting its rows; the shape is selected per
-// plan (ctr_plan_set_fwd_shape).  The resident-CTA hint keeps 32 warps per SM.
-template <typename S, int SLOTS, int SEGS, bool PAIRS = false>
-__global__ void __launch_bounds__(32 * SLOTS * SEGS, CTR_ORBIT_MINB * ORBIT_SLOTS * ORBIT_SEGS / (SLOTS * SEGS))
-k_forward_orbit(const typename OrbitRec<S>::type *__restrict__ ubar, int n, int n_jobs, int M,
-                const OrbitJob *__restrict__ jobs, ForwardEpi<float> epi)
-{
-    pdl_wait();
-    pdl_trigger();
-    forward_orbit_body<S, false, SEGS, SLOTS, PAIRS>(ubar, n, n_jobs, M, jobs, epi, blockIdx.x, blockIdx.y);
-}
-
-// ---------------------------------------------------------------------------
-// Symmetric forward projector with shared staging (launch shape (4, 1)).  A CTA takes
-// STG_JOBS consecutive jobs -- adjacent canonical angles, whose rays nearly coincide --
-// one warp each, and the same 31 bins.  All warps march the same rows; for every block of
-// STG_ROWS rows the union of the jobs' bands of the orbit image (the pixels their rays
-// cross there) is copied into shared memory with 16-byte cp.async (zero-filled outside the
-// image) while the previous block is marched, so each pixel the group reads comes once from
-// L2 for the four jobs instead of once per job.  Weights, march and sums are those of
-// k_forward_orbit (one warp per job, no row split), so the results equal its shape (1, 1).
-// The window of a block is the union over the jobs of [first pixel of interval kb - 1 on
-// the block's last row, last pixel of interval kb + 30 on its first row]; the plan holds
-// the widest window any block can need (stg_window), which sizes the row pitch.
-// ---------------------------------------------------------------------------
-constexpr int STG_JOBS = 4;
-constexpr int STG_ROWS = 8;
-
-template <typename R>
-__device__ __forceinline__ void cp_async_rec(R *dst, const R *src, bool valid)
-{
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    if constexpr (sizeof(R) == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0)
-                     : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(valid ? 8 : 0)
-                     : "memory");
-}
-
-template <typename S>
-__global__ void __launch_bounds__(32 * STG_JOBS)
-k_forward_orbit_staged(const typename OrbitRec<S>::type *__restrict__ ubar, int n, int n_jobs, int M,
-                       const OrbitJob *__restrict__ jobs, ForwardEpi<float> epi, int wmax, int nst_max)
-{
-    using R = typename OrbitRec<S>::type;
-    constexpr long long ONE = 4294967296ll;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R *stage = reinterpret_cast<R *>(smem_raw);                        // [2][STG_ROWS][wmax]
-    int *s_qlo = reinterpret_cast<int *>(stage + 2 * STG_ROWS * wmax);  // [nst_max]
-    int *s_qhi = s_qlo + nst_max;
-    __shared__ int s_mlo, s_mhi;
-    pdl_wait();
-    pdl_trigger();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int kb = blockIdx.x * 31;
-    const int k = kb + lane - 1;                 // this lane's interval [k, k + 1)
-    const int j0 = blockIdx.y * STG_JOBS;
-    const int nj = min(STG_JOBS, n_jobs - j0);
-    const bool has_job = warp < nj;              // warp-uniform
-    AngleMarch am{};
-    int4 ls = make_int4(-1, -1, -1, -1);
-    if (has_job) {
-        am = jobs[j0 + warp].am;
-        ls = *reinterpret_cast<const int4 *>(jobs[j0 + warp].l);
-    }
-    if (threadIdx.x == 0) {
-        s_mlo = n;
-        s_mhi = -1;
-    }
-    __syncthreads();
-    {   // rows crossed by the CTA's rays on the detector (outer bounds, as k_forward_orbit)
-        int mlo = n, mhi = -1;
-        if (has_job && k < M) {
-            const float Q0 = (float)k * am.kA - am.oA;
-            rows_in<true>(Q0, am.binv, -3.f, (float)n + 1.f, n, mlo, mhi);
-        }
-        mlo = __reduce_min_sync(0xffffffffu, mlo);
-        mhi = __reduce_max_sync(0xffffffffu, mhi);
-        if (lane == 0 && mlo <= mhi) {
-            atomicMin(&s_mlo, mlo);
-            atomicMax(&s_mhi, mhi);
-        }
-    }
-    __syncthreads();
-    const int mlo = s_mlo, mhi = s_mhi;
-    const int nst = mlo <= mhi ? min((mhi - mlo + STG_ROWS) / STG_ROWS, nst_max) : 0;
-    for (int e = threadIdx.x; e < nst; e += blockDim.x) {
-        s_qlo[e] = 0x7fffffff;
-        s_qhi[e] = -0x7fffffff;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < nst * nj; e += blockDim.x) {   // every block's window
-        const int st = e / nj;
-        const AngleMarch a = jobs[j0 + (e - st * nj)].am;
-        const int mf = mlo + st * STG_ROWS, ml = min(mf + STG_ROWS - 1, mhi);
-        const long long lo = ceil_div_ll((long long)(kb - 1) * ONE - (long long)ml * a.B - a.Op, a.A);
-        const long long hi = ceil_div_ll((long long)(kb + 31) * ONE - (long long)mf * a.B - a.Op, a.A) - 1;
-        atomicMin(&s_qlo[st], (int)lo);
-        atomicMax(&s_qhi[st], (int)hi);
-    }
-    __syncthreads();
-    // block st of rows into buffer st & 1: row rr at stage[(st & 1)][rr][c] = pixel q_lo + c
-    auto prefetch = [&](int st) {
-        R *dst = stage + (size_t)(st & 1) * STG_ROWS * wmax;
-        const int q0 = s_qlo[st];
-        const int w = min(s_qhi[st] - q0 + 1, wmax);
-        const int mf = mlo + st * STG_ROWS;
-        const int rows = min(STG_ROWS, mhi - mf + 1);
-        for (int rr = 0; rr < rows; ++rr) {
-            const R *src_row = ubar + (size_t)(mf + rr) * n;
-            for (int c = threadIdx.x; c < w; c += blockDim.x) {
-                const int q = q0 + c;
-                const bool ok = (unsigned)q < (unsigned)n;
-                cp_async_rec(dst + rr * wmax + c, ok ? src_row + q : ubar, ok);
-            }
-        }
-    };
-    float4 Su = make_float4(0.f, 0.f, 0.f, 0.f), Sf = Su;
-    // the lane's march state at row mlo: q = first pixel with P >= K, r = P - K in [0, A)
-    const long long A = am.A > 0 ? am.A : 1, B = am.B;
-    const long long K = (long long)k * ONE;
-    const long long qa = ceil_div_ll(K - (long long)mlo * B - am.Op, A);
-    unsigned r = (unsigned)(qa * A + (long long)mlo * B + am.Op - K);
-    int q = (int)qa;
-    const unsigned A32 = (unsigned)A, B32 = (unsigned)B;
-    const unsigned lim = (unsigned)(ONE - A);
-    // the first pixel moves one to the left when r + B reaches A; with B = 0 it never moves
-    // (and A - B may be 2^32, which a 32-bit threshold cannot hold)
-    const unsigned thr = (unsigned)(A - B);
-    const bool moves = B > 0;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (nst > 0) prefetch(0);
-    cp_async_commit();
-    for (int st = 0; st < nst; ++st) {
-        if (st + 1 < nst) prefetch(st + 1);
-        cp_async_commit();
-        cp_async_wait<1>();                      // this thread's copies of block st
-        __syncthreads();                         // everyone's
-        if (has_job) {
-            const R *blk = stage + (size_t)(st & 1) * STG_ROWS * wmax;
-            const int rows = min(STG_ROWS, mhi - (mlo + st * STG_ROWS) + 1);
-            int idx = q - s_qlo[st];
-#pragma unroll
-            for (int rr = 0; rr < STG_ROWS; ++rr) {
-                if (rr < rows) {
-                    const R *row = blk + rr * wmax;
-                    const float4 v1 = rec_f32(row[idx]);
-                    const float4 v2 = r < lim ? rec_f32(row[idx + 1]) : zero;
-                    acc4(Su, Sf, v1, one_plus_frac32u(r));
-                    acc4(Su, Sf, v2, one_plus_frac32u(r + A32));
-                    const bool sdn = moves && r >= thr;
-                    r += sdn ? B32 - A32 : B32;
-                    idx -= sdn ? 1 : 0;
-                    q -= sdn ? 1 : 0;
-                }
-            }
-        }
-        __syncthreads();                         // buffer st & 1 is refilled next
-    }
-    cp_async_wait<0>();
-    if (!has_job || kb >= M) return;             // warp-uniform
-    orbit_out(epi, j0 + warp, 0, ls.x, M, k, lane, Su.x, Sf.x);
-    orbit_out(epi, j0 + warp, 1, ls.y, M, k, lane, Su.y, Sf.y);
-    orbit_out(epi, j0 + warp, 2, ls.z, M, k, lane, Su.z, Sf.z);
-    orbit_out(epi, j0 + warp, 3, ls.w, M, k, lane, Su.w, Sf.w);
-}
-
-template <typename S>
-void launch_forward_orbit_staged(const ctr_plan *p, const typename OrbitRec<S>::type *ub,
-                                 const ForwardEpi<float> &epi, cudaStream_t s)
-{
-    const dim3 grid(fwd_grid_x(p->M), (p->n_jobs + STG_JOBS - 1) / STG_JOBS);
-    const int rec = (int)sizeof(typename OrbitRec<S>::type);
-    launch_pdl(p->pdl != 0, k_forward_orbit_staged<S>, grid, dim3(32 * STG_JOBS),
-               stg_smem_bytes(p->stg_wmax, p->stg_nst, rec), s, ub, p->n, p->n_jobs, p->M,
-               (const OrbitJob *)p->d_jobs, epi, p->stg_wmax, p->stg_nst);
-}
-
-template <typename S, int SLOTS, int SEGS>
-void launch_forward_orbit_shape(const ctr_plan *p, const typename OrbitRec<S>::type *ub, const ForwardEpi<float> &epi,
-                                cudaStream_t s)
-{
-    const dim3 grid(fwd_grid_x(p->M), (p->n_jobs + SLOTS - 1) / SLOTS);
-    auto kern = k_forward_orbit<S, SLOTS, SEGS, false>;
-    if constexpr (std::is_same<S, float>::value)                  // pair-job variant (two live channels)
-        if (p->pair_jobs) kern = k_forward_orbit<S, SLOTS, SEGS, true>;
-    launch_pdl(p->pdl != 0, kern, grid, dim3(32 * SLOTS * SEGS), 0, s, ub, p->n, p->n_jobs, p->M,
-               (const OrbitJob *)p->d_jobs, epi);
-}
-
-template <typename S>
-void launch_forward_orbit(const ctr_plan *p, const typename OrbitRec<S>::type *ub, const ForwardEpi<float> &epi,
-                          cudaStream_t s)
-{
-    switch (p->fwd_slots * 16 + p->fwd_segs) {
-    case 1 * 16 + 2: launch_forward_orbit_shape<S, 1, 2>(p, ub, epi, s); break;
-    case 1 * 16 + 8: launch_forward_orbit_shape<S, 1, 8>(p, ub, epi, s); break;
-    case 2 * 16 + 2: launch_forward_orbit_shape<S, 2, 2>(p, ub, epi, s); break;
-    case 2 * 16 + 4: launch_forward_orbit_shape<S, 2, 4>(p, ub, epi, s); break;
-    case 4 * 16 + 2: launch_forward_orbit_shape<S, 4, 2>(p, ub, epi, s); break;
-    case 4 * 16 + 1: launch_forward_orbit_staged<S>(p, ub, epi, s); break;
-    default: launch_forward_orbit_shape<S, 1, 4>(p, ub, epi, s); break;
-    }
 }
 
 #include "orbit.cuh"
@@ -1260,17 +801,20 @@ k_orbit_image_batch(const SliceDesc *__restrict__ sd, const int *__restrict__ pr
     orbit_image_body<float>(d.u, d.ubar, d.n, local % tiles, local / tiles);
 }
 
-__global__ void __launch_bounds__(ORBIT_THREADS, CTR_ORBIT_MINB)
+__device__ __forceinline__ OfwArgs ofw_args(const SliceDesc &d)
+{
+    return OfwArgs{d.ubar, d.jobs, d.n, d.M, d.n_jobs, d.job_list[1]};
+}
+
+__global__ void __launch_bounds__(OFW_THREADS, 6)
 k_forward_orbit_batch(const SliceDesc *__restrict__ sd, const int *__restrict__ prefix, int ns)
 {
     const int s = find_slice(prefix, ns, blockIdx.x);
     const SliceDesc &d = sd[s];
     const int local = blockIdx.x - prefix[s];
     if (d.pair_jobs)
-        forward_orbit_body<float, false, ORBIT_SEGS, ORBIT_SLOTS, true>(d.ubar, d.n, d.n_jobs, d.M, d.jobs, d.fwe,
-                                                                       local % d.fwd_chunks, local / d.fwd_chunks);
-    else
-        forward_orbit_body<float>(d.ubar, d.n, d.n_jobs, d.M, d.jobs, d.fwe, local % d.fwd_chunks, local / d.fwd_chunks);
+        ofw_body<2, OFW_JOBS, OFW_SEGS, false>(ofw_args(d), d.fwe, local % d.fwd_chunks, local / d.fwd_chunks);
+    else ofw_body<4, OFW_JOBS, OFW_SEGS, false>(ofw_args(d), d.fwe, local % d.fwd_chunks, local / d.fwd_chunks);
 }
 
 __global__ void __launch_bounds__(FWD_THREADS)
@@ -1341,7 +885,7 @@ ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cud
             }
             p->launches++;
             auto kern = p->pair_jobs ? k_backproject_orbit<2> : k_backproject_orbit<4>;
-            launch_pdl(p->pdl != 0, kern, grid, dim3(OBP_THREADS), obp_smem(p->obp_win, p->pair_jobs ? 2 : 4), s,
+            launch_pdl(p->pdl != 0, kern, grid, dim3(OBP_THREADS), obp_smem(p->pair_jobs ? 2 : 4), s,
                        obp_args(p, bar));
             CTR_CHECK_LAUNCH("k_backproject_orbit");
             if (!defer_reduce) {
@@ -1381,19 +925,19 @@ ctr_status fwd_impl(const ctr_plan *p, const S *u, const S *uT, const ForwardEpi
     const bool exact1 = p->h <= p->ds;
     if constexpr (sizeof(T) == 4) {
         if (p->orbit) {
-            using R = typename OrbitRec<S>::type;
-            R *ub = (R *)p->ubar;
+            float *ub = (float *)p->ubar;
             p->launches++;
             const dim3 og((p->n + 31) / 32, (p->n + 31) / 32);
             if constexpr (std::is_same<S, float>::value) {
-                if (tv) launch_pdl(p->pdl != 0, k_orbit_image_tv, og, dim3(256), 0, s, u, ub, p->n, *tv);
+                if (tv) launch_pdl(p->pdl != 0, k_orbit_image_tv, og, dim3(256), 0, s, u, ub,
+                                   p->n, *tv);
                 else launch_pdl(p->pdl != 0, k_orbit_image<S>, og, dim3(256), 0, s, u, ub, p->n);
             } else {
                 launch_pdl(p->pdl != 0, k_orbit_image<S>, og, dim3(256), 0, s, u, ub, p->n);
             }
             CTR_CHECK_LAUNCH("k_orbit_image");
             p->launches++;
-            launch_forward_orbit<S>(p, ub, epi, s);
+            launch_forward_orbit(p, ub, epi, s);
             CTR_CHECK_LAUNCH("k_forward_orbit");
             return CTR_OK;
         }
@@ -1423,15 +967,10 @@ ctr_status configure_radon(const ctr_plan *p)
     const size_t smem = bp_smem<T>(p);
     ctr_status st = raise_smem_limit(k_backproject<T, T>, smem);
     if (st == CTR_OK && p->orbit)
-        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2>, obp_smem(p->obp_win, 2))
-                          : raise_smem_limit(k_backproject_orbit<4>, obp_smem(p->obp_win, 4));
+        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2>, obp_smem(2), true)
+                          : raise_smem_limit(k_backproject_orbit<4>, obp_smem(4), true);
     if constexpr (sizeof(T) == 4)
         if (st == CTR_OK) st = raise_smem_limit(k_backproject<float, __nv_bfloat16>, smem);
-    if (st == CTR_OK && p->orbit && p->stg_wmax > 0) {
-        st = raise_smem_limit(k_forward_orbit_staged<float>, stg_smem_bytes(p->stg_wmax, p->stg_nst, 16));
-        if (st == CTR_OK)
-            st = raise_smem_limit(k_forward_orbit_staged<__nv_bfloat16>, stg_smem_bytes(p->stg_wmax, p->stg_nst, 8));
-    }
     return st;
 }
 
@@ -1483,54 +1022,28 @@ template bool bp_deferred<double>(const ctr_plan *);
 
 int fwd_grid_x(int M) { return (M + 30) / 31; }
 
-size_t stg_smem_bytes(int wmax, int nst_max, int rec_bytes)
-{
-    return (size_t)2 * STG_ROWS * wmax * rec_bytes + 2 * sizeof(int) * (size_t)nst_max;
-}
+int ofw_batch_groups(const ctr_plan *p) { return ofw_groups(p, OFW_JOBS); }
 
-int stg_blocks_max(int n) { return (n + STG_ROWS) / STG_ROWS + 1; }
-
-// The widest window a staged block can need, over every group of STG_JOBS consecutive jobs:
-// the spread of the jobs' first pixels at equal (K, m) (linear in K and m for each job, so
-// its extremes lie at the corners of the detector x row range) plus the pixels 32 intervals
-// and STG_ROWS - 1 rows span for the steepest job, plus the rounding of both window ends.
-int stg_window(const std::vector<OrbitJob> &jobs, int n, int M)
+int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M)
 {
-    const double one = 4294967296.0;
-    double w = 0.0;
-    for (size_t g = 0; g < jobs.size(); g += STG_JOBS) {
-        const size_t e = std::min(jobs.size(), g + STG_JOBS);
-        double spread = 0.0, span = 0.0;
-        for (double K : {-one, (double)(M + 32) * one})
-            for (double m : {0.0, (double)(n - 1)}) {
-                double lo = 1e300, hi = -1e300;
-                for (size_t j = g; j < e; ++j) {
-                    const double x = (K - m * (double)jobs[j].am.B - (double)jobs[j].am.Op) / (double)jobs[j].am.A;
-                    lo = std::min(lo, x);
-                    hi = std::max(hi, x);
-                }
-                spread = std::max(spread, hi - lo);
-            }
-        for (size_t j = g; j < e; ++j)
-            span = std::max(span, (32.0 * one + (STG_ROWS - 1) * (double)jobs[j].am.B) / (double)jobs[j].am.A);
-        w = std::max(w, std::ceil(spread + span) + 4.0);
+    int most = 1;
+    for (const OrbitJob &j : jobs) {
+        const int nb = (int)((OFW_LANES * j.am.A) >> 32) - 1;
+        most = std::max(most, (M + nb - 1) / nb);
     }
-    return (int)w;
+    return most;
 }
-
-int orbit_fwd_grid_y(int n_jobs) { return (n_jobs + ORBIT_SLOTS - 1) / ORBIT_SLOTS; }
 int fwd_grid_y(int N) { return (N + FWD_AW - 1) / FWD_AW; }
 
-size_t obp_smem_bytes(const ctr_plan *p) { return obp_smem(p->obp_win, p->pair_jobs ? 2 : 4); }
+size_t obp_smem_bytes(const ctr_plan *p) { return obp_smem(p->pair_jobs ? 2 : 4); }
 
-int obp_window(const std::vector<OrbitJob> &jobs, int nc)
+int obp_window(const std::vector<OrbitJob> &jobs)
 {
     // bins of a tile's block centres (30 C + 28 S), two on the left and three on the right,
     // and what the 16-byte alignment of the first bin adds
-    const int al = 4 / nc;
     long long w = 0;
     for (const OrbitJob &j : jobs) w = std::max(w, (30 * j.am.A + 28 * j.am.B) >> 32);
-    return ((int)w + 7 + (al - 1) + al - 1) & ~(al - 1);
+    return std::min(OBP_WIN, ((int)w + 9) & ~1);
 }
 
 template <typename T>
@@ -1555,7 +1068,7 @@ void bp_tiles(int n, int &tx, int &ty)
 ctr_status configure_batch_radon(size_t bp_smem, size_t obp_smem_max)
 {
     ctr_status st = raise_smem_limit(k_backproject_batch, bp_smem);
-    if (st == CTR_OK) st = raise_smem_limit(k_backproject_orbit_batch, obp_smem_max);
+    if (st == CTR_OK) st = raise_smem_limit(k_backproject_orbit_batch, obp_smem_max, true);
     return st;
 }
 
@@ -1568,7 +1081,7 @@ ctr_status launch_batch_radon(int stage, const SliceDesc *sd, const int *prefix,
     case BS_BP: k_backproject_batch<<<blocks, 32 * BP_TY, smem, s>>>(sd, prefix, ns); break;
     case BS_BP_SYM: k_backproject_orbit_batch<<<blocks, OBP_THREADS, smem, s>>>(sd, prefix, ns); break;
     case BS_ORBIT: k_orbit_image_batch<<<blocks, 256, 0, s>>>(sd, prefix, ns); break;
-    case BS_FWD_SYM: k_forward_orbit_batch<<<blocks, ORBIT_THREADS, 0, s>>>(sd, prefix, ns); break;
+    case BS_FWD_SYM: k_forward_orbit_batch<<<blocks, OFW_THREADS, 0, s>>>(sd, prefix, ns); break;
     case BS_FWD: k_forward_batch<<<blocks, FWD_THREADS, 0, s>>>(sd, prefix, ns); break;
     default: return fail(CTR_EINVAL, "not a projector stage");
     }

@@ -673,7 +673,6 @@ void set_ybar(const ctr_plan *p, ForwardEpi<T> &e)
     e.ybar = (T *)p->ybar;
     e.ypitch = p->bar_pitch;
     e.ypad = p->bar_pad;
-    e.ync = p->pair_jobs ? 2 : 4;
     e.yround = p->bf16 ? 1 : 0;
 }
 
@@ -1585,7 +1584,7 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.twist = prm.precond == 2 ? 1 : 0;
         d.n_jobs = p->n_jobs;
         d.jobs = p->d_jobs;
-        d.ubar = (float4 *)p->ubar;
+        d.ubar = (float *)p->ubar;
         d.ybar = (const float *)p->ybar;
         d.bar_pitch = p->bar_pitch;
         d.bar_pad = p->bar_pad;
@@ -1595,7 +1594,7 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.per_group = p->orbit ? (p->n_jobs + p->obp_groups - 1) / p->obp_groups
                                : (p->N + p->bp_groups - 1) / p->bp_groups;
         bp_tiles(p->n, d.bp_tiles_x, d.bp_tiles_y);
-        d.fwd_chunks = fwd_grid_x(p->M);
+        d.fwd_chunks = p->orbit ? p->fwd_chunks : fwd_grid_x(p->M);
         d.rpc = fft_rows_per_cta(p->n);
         d.cw = fft_cols_per_cta(p->n, 4);
         d.packed = batch_slice_packed(b, p);
@@ -1658,7 +1657,8 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         for (int stg = BS_FFT_ROWS; stg <= BS_FFT_ROWS_INV; ++stg)
             if ((r = launch_batch_fft(stg, b->d_desc, pre + stg * stride, ns, b->blocks[stg], b->smem[stg], s)) != CTR_OK) return r;
         for (int stg : {BS_ORBIT, BS_FWD, BS_FWD_SYM})
-            if ((r = launch_batch_radon(stg, b->d_desc, pre + stg * stride, ns, b->blocks[stg], 0, s)) != CTR_OK) return r;
+            if ((r = launch_batch_radon(stg, b->d_desc, pre + stg * stride, ns, b->blocks[stg], b->smem[stg], s)) != CTR_OK)
+                return r;
         if ((r = launch_batch_tv(b->d_desc, pre + BS_TV * stride, ns, b->blocks[BS_TV], s)) != CTR_OK) return r;
         int nl = 0;
         for (int stg = 0; stg < BS_COUNT; ++stg) nl += b->blocks[stg] > 0 ? 1 : 0;
@@ -1740,7 +1740,7 @@ ctr_status batch_prepare(ctr_batch *b)
         cnt[BS_FFT_ROWS_INV] = cnt[BS_FFT_ROWS];
         cnt[BS_ORBIT] = p->orbit ? t32 * t32 : 0;
         cnt[BS_FWD] = p->orbit ? 0 : fwd_grid_x(p->M) * fwd_grid_y(p->N);
-        cnt[BS_FWD_SYM] = p->orbit ? fwd_grid_x(p->M) * orbit_fwd_grid_y(p->n_jobs) : 0;
+        cnt[BS_FWD_SYM] = p->orbit ? p->fwd_chunks * ofw_batch_groups(p) : 0;
         cnt[BS_TV] = grid_for(nn, 256, 1024);
         for (int stg = 0; stg < BS_COUNT; ++stg) pre[(size_t)stg * (ns + 1) + i + 1] = pre[(size_t)stg * (ns + 1) + i] + cnt[stg];
         const size_t smb = p->orbit ? 0 : bp_smem_bytes(p->wstride), smo = p->orbit ? obp_smem_bytes(p) : 0;

@@ -17,9 +17,9 @@ def ct():
     return ctrecon
 
 
-@pytest.mark.parametrize("n,N,M,ds", [(1, 4, 3, 1.0), (2, 2, 1, 1.0), (31, 63, 45, 1.0), (33, 65, 9, 1.0),
+@pytest.mark.parametrize("n,N,M,ds", [(1, 4, 3, 1.0), (2, 4, 1, 1.0), (31, 63, 45, 1.0), (33, 65, 9, 1.0),
                                       (34, 128, 49, 1.0), (66, 130, 400, 1.3), (97, 1030, 138, 1.0),
-                                      (64, 261, 91, 1.9), (36, 1029, 52, 1.0)])
+                                      (64, 261, 91, 1.4), (36, 1029, 52, 1.0)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_matches_oracle(ct, n, N, M, ds, dtype):
     import torch

@@ -21,11 +21,11 @@ THETAS = np.concatenate([[0.0, 1e-9, np.pi / 4, np.arctan(1 / 3), np.arctan(0.5)
 
 
 @pytest.mark.parametrize("n,M,ratio", GEOMETRIES)
-@pytest.mark.parametrize("nc", [4, 2])
-def test_backprojection_windows_and_blocks(n, M, ratio, nc):
+def test_backprojection_windows_and_blocks(n, M, ratio):
     jobs = jobs_of(n, M, THETAS, ratio)
-    al = 4 // nc
-    win = (max((30 * A + 28 * B) >> 32 for A, B, _ in jobs) + 7 + 2 * (al - 1)) // al * al
+    al = 2
+    win = (max((30 * A + 28 * B) >> 32 for A, B, _ in jobs) + 9) & ~1
+    assert win <= 52
     far = (n + 31) // 32 * 32 - 32
     lo, hi = 0, M
     for A, B, Op in jobs:
@@ -75,3 +75,67 @@ def test_backprojection_windows_and_blocks(n, M, ratio, nc):
                         inside = (i < n) & (j < n)
                         want = (1 - w) * at(kk) + w * at(kk + 1)
                         assert np.abs((got - want)[inside]).max(initial=0.0) < 1e-6
+
+
+def rows_out(Q0, binv, qlo, qhi, n):
+    f32 = np.float32
+    if binv != 0:
+        m1, m2 = f32((Q0 - f32(qhi)) * binv), f32((Q0 - f32(qlo)) * binv)
+        a0, a1 = max(0.0, np.floor(min(m1, m2))), min(n - 1.0, np.ceil(max(m1, m2)))
+        return (int(a0), int(a1)) if a0 <= a1 else (n, -1)
+    return (0, n - 1) if qlo < Q0 < qhi else (n, -1)
+
+
+@pytest.mark.parametrize("n,M,ratio", GEOMETRIES + [(40, 300000, 1.0)])
+@pytest.mark.parametrize("segs", [1, 4])
+def test_forward_rows_pads_and_slot_sums(n, M, ratio, segs):
+    lanes, pad, one = 64, 72, 2 ** 32
+    f32 = np.float32
+    u = np.random.default_rng(5).standard_normal((n, n))            # ubar[m][q], one channel
+    qq, mm = np.meshgrid(np.arange(n), np.arange(n))
+    for A, B, Op in jobs_of(n, M, THETAS, ratio):
+        want = np.zeros(M + 2)
+        p = (qq * A + mm * B + Op) / one
+        k = np.floor(p).astype(int)
+        for kk, w in ((k, 1 - (p - k)), (k + 1, p - k)):
+            np.add.at(want, np.where((kk >= 0) & (kk < M), kk + 1, 0), w * u)
+        nb = ((lanes * A) >> 32) - 1
+        assert nb >= 1
+        centre = np.array([-((-q * A) >> 32) for q in range(lanes)])
+        phi = np.array([q * A / one for q in range(lanes)]) - centre
+        chunks = range((M + nb - 1) // nb)
+        for bx in (chunks if M < 1000 else [0, len(chunks) // 2 - 1, len(chunks) // 2, len(chunks) - 1]):
+            kb, S, X, P = bx * nb, np.zeros(lanes), np.zeros(lanes), np.zeros(lanes)
+            K0 = (kb - 1) * one
+            Q0 = f32(K0 - Op) * f32(f32(one / A) * f32(2.0 ** -32))
+            lo, hi = rows_out(Q0, f32(A / B) if B / A > 1e-9 else f32(0), -lanes - 1, n + 1, n)
+            per = (hi - lo + segs) // segs
+            for seg in range(segs):
+                mlo = lo + seg * per
+                mhi = min(hi, mlo + per - 1)
+                if mlo > mhi:
+                    continue
+                q = int(np.ceil(Q0 - f32(mlo) * (f32(B) / f32(A))))
+                x = q * A + mlo * B + Op - K0
+                while x < 0:
+                    x, q = x + A, q + 1
+                while x >= A:
+                    x, q = x - A, q - 1
+                bound = min(A - B, one - 1)
+                r = min(x, one - 2) if B == 0 else x
+                for m in range(mlo, mhi + 1):
+                    assert -pad <= q and q + lanes - 1 < n + pad
+                    assert 0 <= r < A and abs(q * A + m * B + Op - K0 - r) <= (B == 0)
+                    at = np.arange(q, q + lanes)
+                    v = np.where((at >= 0) & (at < n), u[m, np.clip(at, 0, n - 1)], 0.0)
+                    z = r / one + phi
+                    assert np.abs(z).max() <= 1
+                    S, X, P = S + v, X + r / one * v, P + np.clip(z, 0, 1) * v
+                    step = r >= bound
+                    r = (r + (B - A if step else B)) % one
+                    q -= step
+            N = P - X - phi * S
+            got = [P[centre == b].sum() + (S - P - N)[centre == b + 1].sum() + N[centre == b + 2].sum()
+                   for b in range(min(nb, M - kb))]
+            ref = want[1:-1][kb:min(kb + nb, M)]
+            assert np.abs(np.array(got) - ref).max(initial=0.0) < 1e-4 * max(1.0, np.abs(want[1:-1]).max())
