@@ -15,8 +15,8 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libctrecon.so")
 ROOT = os.path.dirname(HERE)
 HEADERS = [os.path.join(ROOT, "include", "ctrecon.h"), os.path.join(SRC, "ctr_internal.cuh")]
-# kernels.cu includes radon.cu (which includes orbit.cuh) and fft.cu: one translation unit, see its header
-INCLUDED = {"kernels.cu": ["radon.cu", "fft.cu", "orbit.cuh"]}
+# kernels.cu includes radon.cu (which includes orbit.cuh and orbit64.cuh) and fft.cu: one translation unit, see its header
+INCLUDED = {"kernels.cu": ["radon.cu", "fft.cu", "orbit.cuh", "orbit64.cuh"]}
 UNITS = ["kernels.cu", "solver.cu", "capi.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -109,7 +109,30 @@ long long floor_div2(__int128 v)
     return (long long)q;
 }
 
-// Groups the angles of an FP32 plan into the forward projector's symmetric jobs
+// The tables and buffers of an FP64 plan on the symmetric path: its job groups (tiles of 16 x 16
+// pixels x groups of about 1216 CTAs of two warps, two jobs or more each) leave partial planes.
+ctr_status build_sym64(ctr_plan *p, const std::vector<OrbitJob> &jobs)
+{
+    const size_t nn = (size_t)p->n * p->n;
+    ctr_status st;
+    void *tmp = nullptr;
+    if ((st = alloc(p, &tmp, sizeof(OrbitJob) * jobs.size())) != CTR_OK) return st;
+    p->d_jobs = (OrbitJob *)tmp;
+    CTR_CUDA(cudaMemcpy(p->d_jobs, jobs.data(), sizeof(OrbitJob) * jobs.size(), cudaMemcpyHostToDevice));
+    if ((st = alloc(p, &p->ubar, sym64_image_bytes(p->n))) != CTR_OK) return st;
+    CTR_CUDA(cudaMemset(p->ubar, 0, sym64_image_bytes(p->n)));     // the pads stay zero
+    const int tiles = ((p->n + 15) / 16) * ((p->n + 15) / 16);
+    const int most = std::max(1, (int)jobs.size() / (p->pair_jobs ? 4 : 2));
+    p->bp_groups = std::min(std::min((1216 + tiles - 1) / tiles, MAX_BP_GROUPS), most);
+    p->bp_cap = std::max(p->bp_cap, p->bp_groups);
+    if ((st = alloc(p, &p->bp_part, sizeof(double) * 4 * nn * p->bp_cap)) != CTR_OK) return st;
+    p->n_jobs = (int)jobs.size();
+    p->fwd_chunks = orbit_fwd_chunks(jobs, p->M, p->F);
+    p->sym64 = true;
+    return CTR_OK;
+}
+
+// Groups the angles of a plan into the forward projector's symmetric jobs
 // (OrbitJob): every angle's (C, S) must be one of (a, b), (-a, b), (b, a), (-b, a) of
 // its canonical pair a = max(|C|, |S|), b = min(|C|, |S|) (true for angles in
 // [0, pi)); angles with equal canonical pairs share a job, one per channel.  The
@@ -142,28 +165,35 @@ bool shape41_fits(const std::vector<OrbitJob> &jobs, int n, int M)
 
 ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
 {
-    const int n = p->n, N = p->N, M = p->M;
+    const int n = p->n, N = p->N, M = p->M, F = p->F;
+    const long long one = 1ll << F;
+    // FP64: cos and sin of mirrored angles may differ in their last bit, so that equal pairs
+    // come out up to a few units of 2^-F apart; such angles share a job where the shift stays
+    // within half a unit of 2^-48, the resolution the FP64 geometry is specified to
+    const long long tol = F >= 49 ? 1ll << (F - 49) : 0;
     std::vector<OrbitJob> jobs;
     std::map<std::pair<long long, long long>, std::vector<int>> by_pair;   // canonical pair -> jobs
     for (int l = 0; l < N; ++l) {
         const long long C = geo[l].C, S = geo[l].S;
         const long long aC = C < 0 ? -C : C, aS = S < 0 ? -S : S;
         const long long a = aC >= aS ? aC : aS, b = aC >= aS ? aS : aC;
-        // the symmetric kernels track 32-bit remainders and step at most one bin per row:
-        // 1 <= a <= 2^32 (h <= ds makes it so; anything else takes the per-angle path)
-        if (a < 1 || a > (1ll << 32)) return CTR_OK;
+        // the symmetric kernels track remainders in F bits and step at most one bin per row:
+        // 1 <= a <= 2^F (h <= ds makes it so; anything else takes the per-angle path)
+        if (a < 1 || a > one) return CTR_OK;
         const long long img[4][2] = {{a, b}, {-a, b}, {b, a}, {-b, a}};
         bool placed = false, member = false;
-        std::vector<int> &js = by_pair[{a, b}];
         for (int v = 0; v < 4 && !placed; ++v) {
             if (img[v][0] != C || img[v][1] != S) continue;
             member = true;
-            for (int j : js)
-                if (jobs[j].l[v] < 0) {
-                    jobs[j].l[v] = l;
-                    placed = true;
-                    break;
-                }
+            for (auto it = by_pair.lower_bound({a - tol, 0}); it != by_pair.end() && it->first.first <= a + tol && !placed; ++it) {
+                if (it->first.second < b - tol || it->first.second > b + tol) continue;
+                for (int j : it->second)
+                    if (jobs[j].l[v] < 0) {
+                        jobs[j].l[v] = l;
+                        placed = true;
+                        break;
+                    }
+            }
         }
         if (!member) return CTR_OK;                 // outside the symmetric set: per-angle path
         if (!placed) {
@@ -174,14 +204,14 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
             am.flip = 0;
             am.A = a;
             am.B = b;
-            am.Op = floor_div2(((__int128)(M - 1) << 32) - (__int128)(n - 1) * ((__int128)a + (__int128)b));
-            am.kA = (float)(4294967296.0 / (double)a);
+            am.Op = floor_div2(((__int128)(M - 1) << F) - (__int128)(n - 1) * ((__int128)a + (__int128)b));
+            am.kA = (float)((double)one / (double)a);
             am.oA = (float)((double)am.Op / (double)a);
             const double bA = (double)b / (double)a;
             am.binv = bA > 1e-9 ? (float)(1.0 / bA) : 0.f;
             for (int v = 0; v < 4; ++v)
                 if (img[v][0] == C && img[v][1] == S) { jb.l[v] = l; break; }
-            js.push_back((int)jobs.size());
+            by_pair[{a, b}].push_back((int)jobs.size());
             jobs.push_back(jb);
         }
     }
@@ -194,7 +224,7 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
             if ((jb.l[2] < 0 && jb.l[3] < 0) || (jb.l[0] < 0 && jb.l[1] < 0)) ++pairs;
         p->pair_jobs = 2 * pairs > jobs.size() ? 1 : 0;
     }
-    p->shape41 = shape41_fits(jobs, n, M);
+    if (F == 32) p->shape41 = shape41_fits(jobs, n, M);
     // the job lists: one, or the pair jobs of channels {0, 1} and those of {2, 3} (a job with
     // angles in both becomes two); each sorted by S / C, so that neighbours' rays nearly coincide
     {
@@ -218,6 +248,7 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
             p->job_list[h + 1] = (int)jobs.size();
         }
     }
+    if (F != 32) return build_sym64(p, jobs);
     const int nc = p->pair_jobs ? 2 : 4;
     {
         // orbit-layout rows: every tile's window of obp_win bins, and the detector, inside the row
@@ -238,7 +269,7 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     p->d_jobs = (OrbitJob *)tmp;
     if ((st = alloc(p, &p->ubar, sizeof(float4) * (size_t)n * orbit_pitch(n))) != CTR_OK) return st;
     CTR_CUDA(cudaMemset(p->ubar, 0, sizeof(float4) * (size_t)n * orbit_pitch(n)));   // the pads stay zero
-    p->fwd_chunks = orbit_fwd_chunks(jobs, M);
+    p->fwd_chunks = orbit_fwd_chunks(jobs, M, F);
     // the symmetric backprojection: job groups so that tiles x groups is about 1024 CTAs
     // (~1.7 waves of 4 eight-warp CTAs per SM on 152 SMs; measured best at n = 512 among
     // 2..8), at least 8 jobs per group; room for up to MAX_BP_GROUPS groups at n <= 1024
@@ -309,7 +340,7 @@ ctr_status build_tables(ctr_plan *p)
     p->wstride = (int)wmax;
     CTR_CUDA(cudaMemcpy(p->d_geom, geo.data(), sizeof(AngleGeom) * N, cudaMemcpyHostToDevice));
     CTR_CUDA(cudaMemcpy(p->d_march, mar.data(), sizeof(AngleMarch) * N, cudaMemcpyHostToDevice));
-    if (p->F == 32 && p->h <= p->ds && ncand == 2) return build_orbit_jobs(p, geo);
+    if (p->h <= p->ds && ncand == 2) return build_orbit_jobs(p, geo);
     return CTR_OK;
 }
 
@@ -557,7 +588,7 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
     p->theta.assign(g->angles_host, g->angles_host + g->n_angles);
     if (dtype == CTR_F64) {
         int F = 62 - (int)std::ceil(std::log2(pmax));
-        p->F = F > 48 ? 48 : F;
+        p->F = F > 51 ? 51 : F;
         p->esize = 8;
     } else {
         p->F = 32;
@@ -673,7 +704,8 @@ ctr_status rh_forward(ctr_plan *p, const void *u, void *g, void *stream)
     cudaStream_t s = (cudaStream_t)stream;
     ctr_status st;
     if (p->dtype == CTR_F64) {
-        if ((st = launch_transpose<double>(p, (const double *)u, (double *)p->uT, s)) != CTR_OK) return st;
+        if (fwd_needs_transpose<double>(p) && (st = launch_transpose<double>(p, (const double *)u, (double *)p->uT, s)) != CTR_OK)
+            return st;
         return op_forward<double>(p, (const double *)u, (const double *)p->uT, (double *)g, 1.0, s);
     }
     if (p->bf16) {

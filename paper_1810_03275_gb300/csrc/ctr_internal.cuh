@@ -102,7 +102,7 @@ template <> struct Cplx<double> { using type = double2; };
 // grid is centred.  floor(p) = P >> F and frac(p) = (P mod 2^F) 2^-F.  Both
 // projectors derive every interpolation weight from the same integer P, so the
 // ray-driven R_h is the exact transpose of the pixel-driven R_h^*.
-// F = 32 for FP32/BF16 (weight = top 23 fraction bits), F = 48 or less for FP64.
+// F = 32 for FP32/BF16 (weight = top 23 fraction bits), F = 51 or less for FP64 (48 at 4096^2).
 // ---------------------------------------------------------------------------
 struct AngleGeom {
     long long C, S, O;
@@ -181,13 +181,14 @@ __device__ __forceinline__ T bp_epilogue_value(const BackprojEpi<T> &epi, int n,
 
 // The fold of the symmetric backprojection (OrbitJob path): its partial planes
 // [group][v][row][col] summed at image pixel (i, j) in a fixed order.
-__device__ __forceinline__ float orbit_fold(const float *__restrict__ part, int groups, int n, int i, int j)
+template <typename T>
+__device__ __forceinline__ T orbit_fold(const T *__restrict__ part, int groups, int n, int i, int j)
 {
     const size_t nn = (size_t)n * n;
     const size_t e = (size_t)i * n + j, em = (size_t)(n - 1 - i) * n + j;
-    float s = 0.f;
+    T s = T(0);
     for (int z = 0; z < groups; ++z) {
-        const float *pz = part + (size_t)z * 4 * nn;
+        const T *pz = part + (size_t)z * 4 * nn;
         s += pz[e] + pz[nn + em] + pz[2 * nn + e] + pz[3 * nn + em];
     }
     return s;
@@ -401,6 +402,7 @@ struct ctr_plan {
     ctr::AngleGeom *d_geom = nullptr;
     ctr::AngleMarch *d_march = nullptr;
     bool orbit = false;                  // FP32 forward projector on the symmetric path
+    bool sym64 = false;                  // FP64 plan on the symmetric path (jobs in 2^-F bins, partial planes in bp_part)
     int n_jobs = 0;
     ctr::OrbitJob *d_jobs = nullptr;
     void *ubar = nullptr;                // orbit image: two planes of n rows of orbit_pitch pixels, 8 bytes each
@@ -524,10 +526,11 @@ int backproject_tile_rows();   // pixel rows of a backprojection tile (its width
 template <typename T> bool bp_deferred(const ctr_plan *p);
 // false when the forward projector reads only u (the symmetric path builds its own
 // orbit image): callers may then skip making the transposed copy uT
-template <typename T> inline bool fwd_needs_transpose(const ctr_plan *p) { return !(sizeof(T) == 4 && p->orbit); }
+template <typename T> inline bool fwd_needs_transpose(const ctr_plan *p) { return !(sizeof(T) == 4 && p->orbit) && !p->sym64; }
 int fwd_grid_x(int M);         // forward-projector grid: bin chunks
 int ofw_batch_groups(const ctr_plan *p);        // symmetric forward projector, batched stage: groups of jobs
-int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M);   // symmetric forward projector: bin chunks per job
+int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M, int F);
+size_t sym64_image_bytes(int n);     // orbit image of an FP64 plan   // symmetric forward projector: bin chunks per job
 // its pixels per warp and row, and the zero pixels on either side of an orbit-image row (every
 // read of the march lies within them)
 constexpr int OFW_LANES = 64, ORBIT_PAD = OFW_LANES + 8;

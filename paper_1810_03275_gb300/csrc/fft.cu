@@ -244,7 +244,7 @@ struct RowsInput {
     const T *in_real;
     const T *part;
     int groups;
-    int orbit;                // part holds the symmetric path's partial planes (FP32)
+    int orbit;                // part holds the symmetric path's partial planes
     BackprojEpi<T> epi;
 };
 
@@ -255,10 +255,9 @@ __device__ __forceinline__ T rows_input_value(const RowsInput<T> &src, int n, in
     const size_t e = (size_t)row * n + col;
     if (!src.part) return src.in_real[e];
     T acc;
-    if constexpr (sizeof(T) == 4) {
-        if (src.orbit) acc = orbit_fold(src.part, src.groups, n, row, col);
-    }
-    if (!(sizeof(T) == 4 && src.orbit)) {
+    if (src.orbit) {
+        acc = orbit_fold(src.part, src.groups, n, row, col);
+    } else {
         const size_t nn = (size_t)n * n;
         const T *pp = src.part + e;
         acc = pp[0];
@@ -374,10 +373,9 @@ __device__ __forceinline__ void fft_rows_fwd_body(const RowsInput<T> &src, typen
         staged_copy(cnt * n, [&](int e) {
             const int di = fast_div(e, n, mn);
             T acc;
-            if constexpr (sizeof(T) == 4) {
-                if (src.orbit) acc = orbit_fold(src.part, src.groups, n, r0 + di, e - di * n);
-            }
-            if (!(sizeof(T) == 4 && src.orbit)) {
+            if (src.orbit) {
+                acc = orbit_fold(src.part, src.groups, n, r0 + di, e - di * n);
+            } else {
                 const T *pp = src.part + g0 + e;
                 acc = pp[0];
 #pragma unroll
@@ -1194,9 +1192,10 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
     p->launches++;
     RowsInput<T> src{};
     if (bp_in) {
-        src.orbit = sizeof(T) == 4 && p->orbit;
-        src.part = (const T *)(src.orbit ? p->obp_part : p->bp_part);
-        src.groups = src.orbit ? p->obp_groups : p->bp_groups;
+        const bool orbit32 = sizeof(T) == 4 && p->orbit;
+        src.orbit = orbit32 || p->sym64;
+        src.part = (const T *)(orbit32 ? p->obp_part : p->bp_part);
+        src.groups = orbit32 ? p->obp_groups : p->bp_groups;
         src.epi = *bp_in;
     } else if (!in_is_cbuf) {
         src.in_real = in_real;

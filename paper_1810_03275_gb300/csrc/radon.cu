@@ -734,18 +734,20 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c)
 }
 
 #include "orbit.cuh"
+#include "orbit64.cuh"
 
 // The fold of the symmetric backprojection's partial planes, then the
 // backprojection epilogue (grid-stride over the pixels).
+template <typename T>
 __global__ void __launch_bounds__(256)
-k_bp_fold(const float *__restrict__ part, int groups, int n, BackprojEpi<float> epi)
+k_bp_fold(const T *__restrict__ part, int groups, int n, BackprojEpi<T> epi)
 {
     pdl_wait();
     pdl_trigger();
     const size_t nn = (size_t)n * n;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nn; e += (size_t)gridDim.x * blockDim.x) {
         const int i = pix_i(e, n), j = pix_j(e, n);
-        bp_epilogue(epi, n, i, j, orbit_fold(part, groups, n, i, j));
+        bp_epilogue(epi, n, i, j, orbit_fold<T>(part, groups, n, i, j));
     }
 }
 
@@ -893,9 +895,21 @@ ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cud
                 int blocks = (int)((nn + 255) / 256);
                 if (blocks > 4096) blocks = 4096;
                 p->launches++;
-                launch_pdl(p->pdl != 0, k_bp_fold, dim3(blocks), dim3(256), 0, s, (const float *)part, G, p->n, epi);
+                launch_pdl(p->pdl != 0, k_bp_fold<float>, dim3(blocks), dim3(256), 0, s, (const float *)part, G, p->n, epi);
                 CTR_CHECK_LAUNCH("k_bp_fold");
             }
+            return CTR_OK;
+        }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        if (p->sym64) {
+            ctr_status st = launch_backproject_sym64(p, g, s);
+            if (st != CTR_OK || defer_reduce) return st;
+            const size_t nn = (size_t)p->n * p->n;
+            p->launches++;
+            k_bp_fold<double><<<(int)std::min<size_t>((nn + 127) / 128, 4096), 128, 0, s>>>((const double *)p->bp_part,
+                                                                                          p->bp_groups, p->n, epi);
+            CTR_CHECK_LAUNCH("k_bp_fold");
             return CTR_OK;
         }
     }
@@ -942,6 +956,8 @@ ctr_status fwd_impl(const ctr_plan *p, const S *u, const S *uT, const ForwardEpi
             return CTR_OK;
         }
     }
+    if constexpr (std::is_same<T, double>::value)
+        if (p->sym64) return launch_forward_sym64(p, u, epi, s);
     p->launches++;
     dim3 grid(fwd_grid_x(p->M), fwd_grid_y(p->N));
     switch (p->ncand * 2 + (exact1 ? 1 : 0)) {
@@ -1015,7 +1031,7 @@ int backproject_tile_rows() { return BP_TI; }
 template <typename T>
 bool bp_deferred(const ctr_plan *p)
 {
-    return p->bp_groups > 1 || (sizeof(T) == 4 && p->orbit);
+    return p->bp_groups > 1 || (sizeof(T) == 4 && p->orbit) || p->sym64;
 }
 template bool bp_deferred<float>(const ctr_plan *);
 template bool bp_deferred<double>(const ctr_plan *);
@@ -1024,11 +1040,14 @@ int fwd_grid_x(int M) { return (M + 30) / 31; }
 
 int ofw_batch_groups(const ctr_plan *p) { return ofw_groups(p, OFW_JOBS); }
 
-int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M)
+size_t sym64_image_bytes(int n) { return 2 * sizeof(double2) * (size_t)n * f64_pitch(n); }
+
+int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M, int F)
 {
+    const int lanes = F == 32 ? OFW_LANES : F64_LANES;
     int most = 1;
     for (const OrbitJob &j : jobs) {
-        const int nb = (int)((OFW_LANES * j.am.A) >> 32) - 1;
+        const int nb = (int)((lanes * j.am.A) >> F) - 1;
         most = std::max(most, (M + nb - 1) / nb);
     }
     return most;
