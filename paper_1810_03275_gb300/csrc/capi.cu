@@ -633,7 +633,7 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
     ALLOC(p->ubar_u, es * nn);
     ALLOC(p->pk_s, es * nn);
     ALLOC(p->aux, es * nn);
-    p->ramp_L = ramp_length(p->M);
+    p->ramp_L = ramp_length(p->M, p->esize);
     if ((st = fft_radices(p->ramp_L, p->ramp_radices)) != CTR_OK) {
         destroy(p);
         return st;

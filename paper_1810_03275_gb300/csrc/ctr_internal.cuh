@@ -516,7 +516,7 @@ ctr_status launch_fft2_forward(const ctr_plan *p, const T *in_real, cudaStream_t
 template <typename T> ctr_status configure_radon(const ctr_plan *p);   // smem attributes, at plan creation
 template <typename T> ctr_status configure_fft(const ctr_plan *p);
 ctr_status fft_radices(int n, std::vector<int> &out);
-int ramp_length(int M);   // smallest 2^a 3^b >= 2M - 1
+int ramp_length(int M, size_t esize);   // FFT length of the ramp filter, 2^a 3^b >= 2M - 1
 // y = (ramp-filtered g) * outscale per view (N x M); yh (optional): the same in bfloat16 instead
 template <typename T>
 ctr_status launch_ramp(ctr_plan *p, const T *g, T *y, __nv_bfloat16 *yh, double outscale, cudaStream_t s);
