@@ -599,6 +599,17 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
     ctr_status st = fft_radices(p->n, p->radices);
     p->fft_ok = (st == CTR_OK);
     if (!p->fft_ok) p->radices.clear();
+    if (dtype == CTR_F64 && p->n < 1024) {
+        // FP64: a warp instruction takes 64 cycles of its scheduler however many lanes work, so
+        // a pass is as long as its butterfly and radix 2 keeps the most lanes busy (64^2: a
+        // radix-8 pass has 8 butterflies of about 100 operations, a radix-2 one 32 of 10)
+        std::vector<int> small;
+        for (int r : p->radices)
+            if (r == 3) small.push_back(3);
+            else
+                for (; r > 1; r /= 2) small.push_back(2);
+        if (small.size() <= 16) p->radices = small;
+    }
     st = CTR_OK;
     if (cudaGetDevice(&p->device) != cudaSuccess) { destroy(p); return fail(CTR_ECUDA, "no CUDA device"); }
     const size_t nn = (size_t)p->n * p->n, nm = (size_t)p->N * p->M, es = p->esize;

@@ -52,7 +52,10 @@ struct NvtxScope {
 // completed and its writes are visible (and, since that kernel did the same, every
 // earlier one).  pdl_trigger() lets the next such launch be scheduled as soon as every CTA
 // of this grid is resident, so the launch latency overlaps the tail of this kernel.
-// Both are no-ops for a kernel launched without the attribute.
+// Both are no-ops for a kernel launched without the attribute.  The projectors trigger at
+// their CTAs' ends: triggered at their start, the next kernel's CTAs settle on the SMs that
+// run dry first and stay unevenly spread (Alg. 4, 384^2: 77 us an iteration against 72, 432^2:
+// 93.6 against 87.7, 512^2: 99.7 against 97.3); the short kernels trigger at once.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -187,7 +190,8 @@ __device__ __forceinline__ T orbit_fold(const T *__restrict__ part, int groups, 
     const size_t nn = (size_t)n * n;
     const size_t e = (size_t)i * n + j, em = (size_t)(n - 1 - i) * n + j;
     T s = T(0);
-    for (int z = 0; z < groups; ++z) {
+#pragma unroll 4
+    for (int z = 0; z < groups; ++z) {                               // (the loads of four groups in flight)
         const T *pz = part + (size_t)z * 4 * nn;
         s += pz[e] + pz[nn + em] + pz[2 * nn + e] + pz[3 * nn + em];
     }
@@ -206,6 +210,7 @@ __device__ __forceinline__ float4 orbit_fold4(const float *__restrict__ part, in
     const size_t nn = (size_t)n * n;
     const size_t e = (size_t)i * n + col, em = (size_t)(n - 1 - i) * n + col;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
     for (int z = 0; z < groups; ++z) {
         const float *pz = part + (size_t)z * 4 * nn;
         const float4 a = __ldg(reinterpret_cast<const float4 *>(pz + e));

@@ -8,6 +8,7 @@
 //   columns: forward FFT of a block of columns, multiply by sym, inverse FFT
 //   rows   : inverse FFT of every row, then the epilogue (write, or add to the
 //            iterate and also write its transpose for the ray-driven projector).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -61,6 +62,10 @@ namespace {
 #endif
 constexpr int FFT_THREADS = CTR_FFT_THREADS;
 constexpr int MAX_PASSES = 16;
+#ifndef CTR_FFT_MIN_CTAS
+#define CTR_FFT_MIN_CTAS 128
+#endif
+constexpr int FFT_MIN_CTAS = CTR_FFT_MIN_CTAS;   // CTAs a real-input pass is split into, where it has as many transforms
 
 
 template <typename T> struct C2;
@@ -241,12 +246,21 @@ __device__ __forceinline__ void staged_copy(int total, L load, W store)
     }
 }
 
-// The twiddle table copied into shared memory (read by every pass of the CTA).
+// The twiddle table copied into shared memory (read by every pass of the CTA), asynchronously:
+// it is a constant of the plan, so its copy may run before the kernel ahead has finished.
+// twiddles_ready() before the barrier ahead of the first pass.
 template <typename T2>
 __device__ __forceinline__ void stage_twiddles(T2 *stw, const T2 *__restrict__ tw, int n)
 {
-    for (int t = threadIdx.x; t < n; t += blockDim.x) stw[t] = tw[t];
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const unsigned d = (unsigned)__cvta_generic_to_shared(stw + t);
+        if constexpr (sizeof(T2) == 16)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(tw + t) : "memory");
+        else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(tw + t) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
 }
+__device__ __forceinline__ void twiddles_ready() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Input of the forward row pass.  part != null: the angle-group partial images of
 // the backprojection, summed in group order and passed through the backprojection
@@ -299,6 +313,8 @@ __device__ __forceinline__ void fft_rows_fwd_packed_body(const RowsInput<T> &src
     T2 *b = a + (size_t)cmax * n;
     T2 *stw = b + (size_t)cmax * n;
     stage_twiddles(stw, tw, n);
+    pdl_wait();
+    pdl_trigger();
     const int r0 = bx * rows_per_cta;
     const int cnt = min(rows_per_cta, n - r0);
     const int cc = (cnt + 1) / 2;
@@ -339,6 +355,7 @@ __device__ __forceinline__ void fft_rows_fwd_packed_body(const RowsInput<T> &src
             v.y = ra + 1 < r0 + cnt ? rows_input_value(src, n, ra + 1, j) : T(0);
             return v;
         }, [&](int e, T2 v) { a[e] = v; });
+    twiddles_ready();
     __syncthreads();
     T2 *res = fft_smem<T>(a, b, n, cc, n, fp, -1, stw);
     const unsigned mh = div_magic(H);
@@ -376,6 +393,8 @@ __device__ __forceinline__ void fft_rows_fwd_body(const RowsInput<T> &src, typen
     T2 *b = a + (size_t)rows_per_cta * n;
     T2 *stw = b + (size_t)rows_per_cta * n;
     stage_twiddles(stw, tw, n);
+    pdl_wait();
+    pdl_trigger();
     const int r0 = bx * rows_per_cta;
     const int cnt = min(rows_per_cta, n - r0);
     const size_t g0 = (size_t)r0 * n;
@@ -410,6 +429,7 @@ __device__ __forceinline__ void fft_rows_fwd_body(const RowsInput<T> &src, typen
     } else {
         staged_copy(cnt * n, [&](int e) { return cbuf[g0 + e]; }, put);
     }
+    twiddles_ready();
     __syncthreads();
     T2 *res = fft_smem<T>(a, b, n, cnt, n, fp, -1, stw);
     staged_copy(cnt * n, [&](int e) { return res[e]; }, [&](int e, T2 v) { cbuf[g0 + e] = v; });
@@ -447,9 +467,22 @@ __device__ __forceinline__ void fft_cols_body(typename C2<T>::type *cbuf, const 
     T2 *b = a + (size_t)cw * ld;
     T2 *stw = b + (size_t)cw * ld;
     stage_twiddles(stw, tw, n);
+    pdl_wait();
+    pdl_trigger();
     const int c0 = bx * cw;
     const int cnt = min(cw, ncols - c0);
     const unsigned mc = div_magic(cnt);
+    // the symbol's values, fetched with the data where a thread holds few of them
+    constexpr int SYM_REGS = 4;
+    const bool sym_ahead = sym && cnt * n <= SYM_REGS * (int)blockDim.x;
+    T sreg[SYM_REGS];
+    if (sym_ahead) {
+#pragma unroll
+        for (int k = 0; k < SYM_REGS; ++k) {
+            const int e = threadIdx.x + k * blockDim.x, row = fast_div(e, cnt, mc);
+            sreg[k] = e < cnt * n ? sym[(size_t)row * n + c0 + (e - row * cnt)] : T(0);
+        }
+    }
     // element e: row e / cnt, column c0 + e % cnt (consecutive threads: consecutive columns)
     staged_copy(cnt * n, [&](int e) {
         const int row = fast_div(e, cnt, mc);
@@ -459,6 +492,7 @@ __device__ __forceinline__ void fft_cols_body(typename C2<T>::type *cbuf, const 
         if (twist) v = cmul(v, twist_factor(T(0), row * (c0 + e - row * cnt), n * n));
         a[(size_t)(e - row * cnt) * ld + row] = v;
     });
+    twiddles_ready();
     __syncthreads();
     T2 *res = fft_smem<T>(a, b, n, cnt, ld, fp, -1, stw);
     if (!sym) {                                   // forward transform only: write F back
@@ -471,15 +505,24 @@ __device__ __forceinline__ void fft_cols_body(typename C2<T>::type *cbuf, const 
         });
         return;
     }
-    staged_copy(cnt * n, [&](int e) {
-        const int row = fast_div(e, cnt, mc);
-        return sym[(size_t)row * n + c0 + (e - row * cnt)];
-    }, [&](int e, T m) {
+    const auto scale = [&](int e, T m) {
         const int row = fast_div(e, cnt, mc);
         T2 &v = res[(size_t)(e - row * cnt) * ld + row];
         v.x *= m;
         v.y *= m;
-    });
+    };
+    if (sym_ahead) {
+#pragma unroll
+        for (int k = 0; k < SYM_REGS; ++k) {
+            const int e = threadIdx.x + k * blockDim.x;
+            if (e < cnt * n) scale(e, sreg[k]);
+        }
+    } else {
+        staged_copy(cnt * n, [&](int e) {
+            const int row = fast_div(e, cnt, mc);
+            return sym[(size_t)row * n + c0 + (e - row * cnt)];
+        }, scale);
+    }
     __syncthreads();
     T2 *other = (res == a) ? b : a;
     T2 *res2 = fft_smem<T>(res, other, n, cnt, ld, fp, +1, stw);
@@ -533,6 +576,8 @@ __device__ __forceinline__ void fft_rows_inv_packed_body(const typename C2<T>::t
     T2 *b = a + (size_t)cmax * n;
     T2 *stw = b + (size_t)cmax * n;
     stage_twiddles(stw, tw, n);
+    pdl_wait();
+    pdl_trigger();
     const int r0 = bx * rows_per_cta;
     const int cnt = min(rows_per_cta, n - r0);
     const int cc = (cnt + 1) / 2;
@@ -557,6 +602,7 @@ __device__ __forceinline__ void fft_rows_inv_packed_body(const typename C2<T>::t
         z.y = xa.y + xb.x;
         return z;
     }, [&](int e, T2 v) { a[e] = v; });
+    twiddles_ready();
     __syncthreads();
     T2 *res = fft_smem<T>(a, b, n, cc, n, fp, +1, stw);
     T *fin = reinterpret_cast<T *>(res == a ? b : a);              // final values, [local row][col]
@@ -608,10 +654,13 @@ __device__ __forceinline__ void fft_rows_inv_body(const typename C2<T>::type *__
     T2 *b = a + (size_t)rows_per_cta * n;
     T2 *stw = b + (size_t)rows_per_cta * n;
     stage_twiddles(stw, tw, n);
+    pdl_wait();
+    pdl_trigger();
     const int r0 = bx * rows_per_cta;
     const int cnt = min(rows_per_cta, n - r0);
     const size_t g0 = (size_t)r0 * n;
     staged_copy(cnt * n, [&](int e) { return cbuf[g0 + e]; }, [&](int e, T2 v) { a[e] = v; });
+    twiddles_ready();
     __syncthreads();
     T2 *res = fft_smem<T>(a, b, n, cnt, n, fp, +1, stw);
     // row-major outputs
@@ -1163,15 +1212,19 @@ int cols_per_cta(const ctr_plan *p) { return fft_cols_per_cta(p->n, p->esize); }
 #ifndef CTR_PACK_COLS_MUL
 #define CTR_PACK_COLS_MUL 1
 #endif
+// (a small image is spread over as many CTAs as it has transforms: the passes are bound by the
+// latency of one CTA's chain, in FP64 by its SM's two FP64 lanes.  FP64 64^2 with the fold, the
+// column pass and the inverse: 32, 15.5 and 10.5 us on 4, 9 and 4 CTAs)
 int packed_rows_per_cta(const ctr_plan *p)
 {
-    return 2 * CTR_PACK_ROWS_MUL * (fft_rows_per_cta(p->n) > 1 ? fft_rows_per_cta(p->n) / 2 : 1);
+    const int pairs = fft_rows_per_cta(p->n) > 1 ? fft_rows_per_cta(p->n) / 2 : 1;
+    return 2 * CTR_PACK_ROWS_MUL * std::max(1, std::min(pairs, p->n / 2 / FFT_MIN_CTAS));
 }
 int packed_cols_per_cta(const ctr_plan *p)
 {
     int c = CTR_PACK_COLS_MUL * (cols_per_cta(p) > 1 ? cols_per_cta(p) / 2 : 1);
     while (c > 1 && 2 * (size_t)c * (p->n + 1) * 2 * p->esize > 160 * 1024) c /= 2;
-    return c;
+    return std::max(1, std::min(c, (p->n / 2 + 1) / FFT_MIN_CTAS));
 }
 size_t packed_rows_smem(const ctr_plan *p) { return (2 * (size_t)(packed_rows_per_cta(p) / 2) * p->n + p->n) * 2 * p->esize; }
 size_t packed_cols_smem(const ctr_plan *p) { return (2 * (size_t)packed_cols_per_cta(p) * (p->n + 1) + p->n) * 2 * p->esize; }
@@ -1232,14 +1285,15 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
         const int prp = packed_rows_per_cta(p), pcw = packed_cols_per_cta(p);
         const int pgr = (n + prp - 1) / prp, pgc = (n / 2 + 1 + pcw - 1) / pcw;
         const size_t psr = packed_rows_smem(p), psc = packed_cols_smem(p);
-        k_fft_rows_fwd_packed<T><<<pgr, FFT_THREADS, psr, s>>>(src, cb, n, prp, fp, tw);
+        const bool pdl = p->pdl != 0 && pgr <= 304;    // (more CTAs crowd on the SMs that run dry first: 768^2 264 us against 246)
+        launch_pdl(pdl, k_fft_rows_fwd_packed<T>, dim3(pgr), dim3(FFT_THREADS), psr, s, src, cb, n, prp, fp, tw);
         CTR_CHECK_LAUNCH("k_fft_rows_fwd_packed");
         p->launches++;
-        k_fft_cols_packed<T><<<pgc, FFT_THREADS, psc, s>>>(cb, sym, n, pcw, fp, tw);
+        launch_pdl(pdl, k_fft_cols_packed<T>, dim3(pgc), dim3(FFT_THREADS), psc, s, cb, sym, n, pcw, fp, tw);
         CTR_CHECK_LAUNCH("k_fft_cols_packed");
         p->launches++;
-        k_fft_rows_inv_packed<T><<<pgr, FFT_THREADS, psr, s>>>(cb, n, prp, fp, tw, out, mode, outT, dout, outh,
-                                                               outTh);
+        launch_pdl(pdl, k_fft_rows_inv_packed<T>, dim3(pgr), dim3(FFT_THREADS), psr, s, (const T2 *)cb, n, prp, fp, tw, out,
+                   mode, outT, dout, outh, outTh);
         CTR_CHECK_LAUNCH("k_fft_rows_inv_packed");
         return CTR_OK;
     }
@@ -1329,6 +1383,7 @@ k_ramp_filter(const T *__restrict__ g, int N, int M, int L, FftPasses fp, const 
             v.y = together && k < M ? g[r0 + M + k] : T(0);
             a[k] = v;
         }
+        twiddles_ready();
         __syncthreads();
         T2 *res = fft_smem<T>(a, b, L, 1, L, fp, -1, stw);
         for (int k = threadIdx.x; k < L; k += FFT_THREADS) {

@@ -309,8 +309,8 @@ template <int NC>
 __global__ void __launch_bounds__(OBP_THREADS, 5) k_backproject_orbit(ObpArgs a)
 {
     pdl_wait();
-    pdl_trigger();
     obp_body<NC, false>(a, blockIdx.x, blockIdx.y, blockIdx.z);
+    pdl_trigger();
 }
 
 size_t obp_smem(int nc)
@@ -536,10 +536,10 @@ __global__ void __launch_bounds__(32 * JOBS * SEGS, 24 / (JOBS * SEGS))
 k_forward_orbit(OfwArgs a, ForwardEpi<float> epi)
 {
     pdl_wait();
-    pdl_trigger();
     // chunks from the detector's middle outwards: the long rays first, the short ones fill the tail
     const int c = blockIdx.y, mid = (gridDim.y - 1) / 2;
     ofw_body<NC, JOBS, SEGS, false>(a, epi, c & 1 ? mid + (c + 1) / 2 : mid - c / 2, blockIdx.x);
+    pdl_trigger();
 }
 
 // CTA rows of the job lists in groups of `jobs`

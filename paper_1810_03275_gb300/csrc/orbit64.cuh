@@ -38,6 +38,7 @@ k_backproject_sym64(const double *__restrict__ g, Sym64Args a, double *__restric
     __shared__ long long s_P[S64_JCH], s_C[S64_JCH], s_S[S64_JCH];
     __shared__ int s_k[S64_JCH];
     __shared__ int s_l[S64_JCH][NC];
+    pdl_wait();
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int i0 = blockIdx.y * S64_TILE, j0 = blockIdx.x * S64_TILE, n = a.n;
     const size_t nn = (size_t)n * n;
@@ -102,6 +103,7 @@ k_backproject_sym64(const double *__restrict__ g, Sym64Args a, double *__restric
             }
         }
     }
+    pdl_trigger();
 }
 
 // ---------------------------------------------------------------------------
@@ -116,6 +118,8 @@ __global__ void __launch_bounds__(256)
 k_orbit_image64(const double *__restrict__ u, double *__restrict__ ubar, int n)
 {
     __shared__ double tC[32][33], tD[32][33];
+    pdl_wait();
+    pdl_trigger();
     const int pitch = n + 2 * F64_PAD;
     const size_t plane = (size_t)pitch * n;
     double2 *ub = reinterpret_cast<double2 *>(ubar) + F64_PAD;
@@ -150,6 +154,7 @@ k_forward_sym64(const double *__restrict__ ubar, Sym64Args a, ForwardEpi<double>
     constexpr int LN = F64_LANES, NT = 32 * F64_SEGS;
     __shared__ double s_part[F64_SEGS][NC][3 * LN];   // the slots' sums for bins c, c + 1, c - 1
     __shared__ int s_first[LN + 4];
+    pdl_wait();
     const int seg = threadIdx.x >> 5, lane = threadIdx.x & 31, jb = blockIdx.y, F = a.F;
     const int half = NC == 4 || jb < a.list[1] ? 0 : 2;
     const long long one = 1ll << F;
@@ -237,6 +242,7 @@ k_forward_sym64(const double *__restrict__ ubar, Sym64Args a, ForwardEpi<double>
         for (int q = s_first[b + 2]; q < s_first[b + 3]; ++q) g += acc[2 * LN + q];
         forward_epilogue<double>(epi, (size_t)l * a.M + k, g);
     }
+    pdl_trigger();
 }
 
 Sym64Args sym64_args(const ctr_plan *p)
@@ -249,8 +255,10 @@ ctr_status launch_backproject_sym64(const ctr_plan *p, const double *g, cudaStre
     p->launches++;
     const int tiles = (p->n + S64_TILE - 1) / S64_TILE;
     const dim3 grid(tiles, tiles, p->bp_groups);
-    if (p->pair_jobs) k_backproject_sym64<2><<<grid, S64_THREADS, 0, s>>>(g, sym64_args(p), (double *)p->bp_part);
-    else k_backproject_sym64<4><<<grid, S64_THREADS, 0, s>>>(g, sym64_args(p), (double *)p->bp_part);
+    // launched early, several CTAs per SM would crowd on those SMs that the kernel ahead leaves
+    // first, and FP64 work does not move (128^2: 144 us an iteration against 118)
+    launch_pdl(p->pdl != 0 && grid.x * grid.y * grid.z <= 152, p->pair_jobs ? k_backproject_sym64<2> : k_backproject_sym64<4>, grid, dim3(S64_THREADS), 0, s, g,
+               sym64_args(p), (double *)p->bp_part);
     CTR_CHECK_LAUNCH("k_backproject_sym64");
     return CTR_OK;
 }
@@ -259,11 +267,11 @@ ctr_status launch_forward_sym64(const ctr_plan *p, const double *u, const Forwar
 {
     p->launches += 2;
     const dim3 tiles((p->n + 31) / 32, (p->n + 31) / 32);
-    k_orbit_image64<<<tiles, 256, 0, s>>>(u, (double *)p->ubar, p->n);
+    launch_pdl(p->pdl != 0, k_orbit_image64, tiles, dim3(256), 0, s, u, (double *)p->ubar, p->n);
     CTR_CHECK_LAUNCH("k_orbit_image64");
     const dim3 grid(p->fwd_chunks, p->n_jobs);
-    if (p->pair_jobs) k_forward_sym64<2><<<grid, 32 * F64_SEGS, 0, s>>>((const double *)p->ubar, sym64_args(p), epi);
-    else k_forward_sym64<4><<<grid, 32 * F64_SEGS, 0, s>>>((const double *)p->ubar, sym64_args(p), epi);
+    launch_pdl(p->pdl != 0 && grid.x * grid.y <= 152, p->pair_jobs ? k_forward_sym64<2> : k_forward_sym64<4>, grid, dim3(32 * F64_SEGS), 0, s,
+               (const double *)p->ubar, sym64_args(p), epi);
     CTR_CHECK_LAUNCH("k_forward_sym64");
     return CTR_OK;
 }

@@ -907,8 +907,8 @@ ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cud
             if (st != CTR_OK || defer_reduce) return st;
             const size_t nn = (size_t)p->n * p->n;
             p->launches++;
-            k_bp_fold<double><<<(int)std::min<size_t>((nn + 127) / 128, 4096), 128, 0, s>>>((const double *)p->bp_part,
-                                                                                          p->bp_groups, p->n, epi);
+            launch_pdl(p->pdl != 0, k_bp_fold<double>, dim3((unsigned)std::min<size_t>((nn + 127) / 128, 4096)), dim3(128), 0,
+                       s, (const double *)p->bp_part, p->bp_groups, p->n, epi);
             CTR_CHECK_LAUNCH("k_bp_fold");
             return CTR_OK;
         }

@@ -128,6 +128,8 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_tv_dual(const T *__restrict__ u, int n, T sigma, T tau, T lam, T inv_h, T *v2b, T *y2, T *t2, T *ub)
 {
+    pdl_wait();
+    pdl_trigger();
     tv_dual_body<T>(u, n, sigma, tau, lam, inv_h, v2b, y2, t2, ub, blockIdx.x, gridDim.x);
 }
 
@@ -393,6 +395,11 @@ ctr_status dot2(ctr_plan *p, const T *a, const T *b, size_t len, double *out_dev
 {
     const int nb = grid_for(len, RED_THREADS * 8, p->red_blocks);   // 8 elements per thread: fewer FP64 tree adds
     p->launches++;
+    if (nb == 1) {                                                  // one block's partial is the sum
+        launch_pdl(p->pdl != 0, k_dot2<T>, dim3(1), dim3(RED_THREADS), 0, s, a, b, len, out_dev);
+        CTR_CHECK_LAUNCH("k_dot2");
+        return CTR_OK;
+    }
     launch_pdl(p->pdl != 0, k_dot2<T>, dim3(nb), dim3(RED_THREADS), 0, s, a, b, len, p->d_red);
     p->launches++;
     launch_pdl(p->pdl != 0, k_finalize<2>, dim3(1), dim3(RED_THREADS), 0, s, (const double *)p->d_red, nb, 0u, out_dev);
@@ -745,9 +752,10 @@ ctr_status pdrq_iteration(ctr_plan *p, const IterArgs<T> &a, bool diag, cudaStre
     if (tv_fused) return CTR_OK;
     const size_t nn = (size_t)n * n;
     p->launches++;
-    k_tv_dual<T><<<grid_for(nn, 256, 4096), 256, 0, s>>>((const T *)p->u, n, a.sigma, a.tau, a.lam, a.inv_h,
-                                                        (T *)p->v2b, (T *)p->y2, diag ? (T *)p->t2 : nullptr,
-                                                        a.nonneg ? (T *)p->ubar_u : nullptr);
+    const int tv_threads = nn < 152 * 256 ? 32 : 256;   // a small image over more SMs (FP64 roots and divisions)
+    launch_pdl(p->pdl != 0, k_tv_dual<T>, dim3(grid_for(nn, tv_threads, 4096)), dim3(tv_threads), 0, s, (const T *)p->u, n,
+               a.sigma, a.tau, a.lam, a.inv_h, (T *)p->v2b, (T *)p->y2, diag ? (T *)p->t2 : (T *)nullptr,
+               a.nonneg ? (T *)p->ubar_u : (T *)nullptr);
     CTR_CHECK_LAUNCH("k_tv_dual");
     return CTR_OK;
 }
