@@ -46,6 +46,11 @@ __device__ __forceinline__ float2 vplane(const Vec<2> &v, int) { return v.a; }
 __device__ __forceinline__ float vget(const Vec<4> &v, int c) { return c == 0 ? v.a.x : c == 1 ? v.a.y : c == 2 ? v.b.x : v.b.y; }
 __device__ __forceinline__ float vget(const Vec<2> &v, int c) { return c == 0 ? v.a.x : v.a.y; }
 
+__device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid)   // zero where not valid
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
 __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
@@ -110,6 +115,10 @@ constexpr int OBP_THREADS = 128;
 constexpr int OBP_JCH = 16;    // jobs per staged chunk (two buffers)
 constexpr int OBP_TJ = 128;    // jobs per table block (one per thread)
 
+// Up to this image size a call stages the sinogram's rows itself instead of having them brought
+// into orbit layout by a kernel of their own (one R_h^* call, 64^2 / 90 views: 12.9 us with it, 9.8
+// without; 256^2 / 360: 14.0, 13.4; 384^2 / 480: 19.5, 20.2; pair jobs 256^2 / 361: 14.5, 15.2)
+constexpr int obp_direct_n(bool pairs) { return pairs ? 192 : 256; }
 constexpr int OBP_WIN = 52;    // bins per staged row (obp_window's most: floor(30 C + 28 S) <= 41, + 9)
 
 // One CTA's inputs (also built from a SliceDesc by the batched stage).
@@ -120,12 +129,14 @@ struct ObpArgs {
     int n, pitch, pad, win; // row pitch and left pad in bins; staged bins per row
     int groups;
     int list[3];            // first job of each list, and the end (NC = 4: one list)
+    const float *g;         // if set: the sinogram itself (N x M), staged from its rows instead of bar
+    int M;
 };
 
 struct ObpTables {
     uint4 *pos;    // {low, high word of the centre of the tile's first block in 2^-31 bins, C, S in 2^-31 bins}
     float4 *e;     // e0 .. e3
-    long long *row;   // first staged bin (element of the orbit layout)
+    long long *row;   // first staged bin (element of the orbit layout; of the detector with ObpArgs::g)
     int *flat;     // number of flat jobs of the table block
 };
 
@@ -213,7 +224,7 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
                 const bool flat = 3 * S <= C;
                 // (e3 = 0 up to rounding either way: both forms of the job then agree)
                 tb.e[tid] = make_float4(0.5f * c + 1.5f * s, 0.5f * c + 0.5f * s, 0.5f * c - 0.5f * s, 0.5f * c - 1.5f * s);
-                tb.row[tid] = (long long)(t0 + tid) * (NC / 2) * a.pitch + first;
+                tb.row[tid] = a.g ? first - a.pad : (long long)(t0 + tid) * (NC / 2) * a.pitch + first;
                 if (tid == 0 && !flat) *tb.flat = 0;
                 if (flat) {                                                // sorted by S / C: the last flat job
                     bool next = false;
@@ -230,6 +241,23 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
             const float2 *bar = reinterpret_cast<const float2 *>(a.bar) + 2 * lane;
             auto prefetch = [&](int ch) {                                  // 16 bytes per lane: win <= 64
                 const int a0 = ch * OBP_JCH, na = min(OBP_JCH, nt - a0);
+                if (a.g) {                                                 // four bytes per lane, zeros off the detector
+                    float *dst = reinterpret_cast<float *>(buf + (ch & 1) * (OBP_JCH * JROW));
+                    for (int t = warp; t < na; t += OBP_THREADS / 32) {
+                        const int4 ls = *reinterpret_cast<const int4 *>(a.jobs[t0 + a0 + t].l);
+                        const int l4[4] = {ls.x, ls.y, ls.z, ls.w};
+                        const int k0 = (int)tb.row[a0 + t];
+                        for (int w = lane; w < a.win; w += 32)
+#pragma unroll
+                            for (int c = 0; c < NC; ++c) {
+                                const int l = NC == 4 || li == 0 ? l4[c] : l4[2 + (c & 1)];
+                                const bool ok = l >= 0 && (unsigned)(k0 + w) < (unsigned)a.M;
+                                cp_async4(dst + 2 * (t * JROW + (c >> 1) * OBP_WIN + w) + (c & 1),
+                                          ok ? a.g + (size_t)l * a.M + k0 + w : a.g, ok);
+                            }
+                    }
+                    return;
+                }
                 float2 *dst = buf + (ch & 1) * (OBP_JCH * JROW) + 2 * lane;
                 if (2 * lane < a.win)
                     for (int t = warp; t < na; t += OBP_THREADS / 32) {
@@ -330,6 +358,7 @@ ObpArgs obp_args(const ctr_plan *p, const float *bar)
     a.pad = p->bar_pad;
     a.win = p->obp_win;
     a.groups = p->obp_groups;
+    a.M = p->M;
     for (int k = 0; k < 3; ++k) a.list[k] = p->job_list[k];
     return a;
 }

@@ -880,15 +880,20 @@ ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cud
             const dim3 grid((p->n + 31) / 32, (p->n + 31) / 32, G);
             float *part = (float *)p->obp_part;
             const float *bar = (const float *)p->ybar;
-            if ((const void *)g != p->ybar) {                              // an operand in sinogram layout
+            const bool plain = (const void *)g != p->ybar;                 // an operand in sinogram layout
+            // small calls are bound by their launches: the kernel stages the rows themselves
+            const bool direct = std::is_same<S, float>::value && plain && p->n <= obp_direct_n(p->pair_jobs != 0);
+            if (plain && !direct) {
                 ctr_status st = launch_orbit_sino<S>(p, g, (float *)p->gbar, s);
                 if (st != CTR_OK) return st;
                 bar = (const float *)p->gbar;
             }
             p->launches++;
             auto kern = p->pair_jobs ? k_backproject_orbit<2> : k_backproject_orbit<4>;
+            ObpArgs args = obp_args(p, bar);
+            if (direct) args.g = (const float *)g;
             launch_pdl(p->pdl != 0, kern, grid, dim3(OBP_THREADS), obp_smem(p->pair_jobs ? 2 : 4), s,
-                       obp_args(p, bar));
+                       args);
             CTR_CHECK_LAUNCH("k_backproject_orbit");
             if (!defer_reduce) {
                 const size_t nn = (size_t)p->n * p->n;
