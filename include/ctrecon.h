@@ -367,21 +367,25 @@ ctr_status ctr_plan_set_fwd_shape(ctr_plan *plan, int jobs_per_cta, int segments
 ctr_status ctr_plan_get_fwd_shape(const ctr_plan *plan, int *jobs_per_cta, int *segments);
 
 /* Tuning hook: the kernels of the Fourier preconditioner passes (Sec. 4.3.1, the 2-D DFT
- * diagonalisation of M).  form 0 [default]: on FP32 plans with n = 256, 512 or 1024 each
- * row pair and each column is one warp's transform (a four-step factorisation n = 32 x
- * n/32 in registers, no CTA barrier); other plans use form 1.  form 1: the CTA-level
+ * diagonalisation of M).  form 0 [default]: on FP32 and BF16 plans with n = 256, 512 or 1024,
+ * and on those with another n = 2^a 3^b from 64 to 864 that is a multiple of 4, each row pair
+ * and each column is one warp's transform (a factorisation n = L V, L, V <= 32, in registers,
+ * no CTA barrier; the second set of sizes where a pass has 16-byte aligned operands and writes
+ * no transposed or BF16 copy); other plans and passes use form 1.  form 1: the CTA-level
  * mixed-radix Stockham passes through shared memory (every n = 2^a 3^b, FP64).  Both
  * compute the same DFT up to FP32 rounding.  CTR_EINVAL for other values.  No allocation;
  * ctr_plan_get_fft_form returns the form the plan's passes take (1 where 0 does not apply). */
 ctr_status ctr_plan_set_fft_form(ctr_plan *plan, int form);
 int ctr_plan_get_fft_form(const ctr_plan *plan);
 
-/* Tuning hook: programmatic dependent launch of the kernels of one iteration on the
- * symmetric FP32 / BF16 path (the backprojection, the three preconditioner passes of form 0,
- * the orbit image with the TV step, the forward projector).  on = 1 [default]: each of them
- * is launched with the programmatic-serialization attribute and waits, before its first
- * global-memory access, for the kernel before it to complete, so its launch overlaps that
- * kernel's last wave; results are identical to on = 0 (plain stream order).  CTR_EINVAL
+/* Tuning hook: programmatic dependent launch of the kernels of one iteration: on the
+ * symmetric FP32 / BF16 / FP64 path the backprojection, the preconditioner passes, the orbit
+ * image with the TV step (FP64: the TV step) and the forward projector; not the FP64
+ * projectors of more than 152 thread blocks nor the form 1 passes of more than 304, which an
+ * early launch slows.  on = 1 [default]: each is launched with the programmatic-serialization
+ * attribute and waits, before its first access to what an earlier kernel writes, for the kernel
+ * before it to complete, so its launch overlaps that kernel's last wave; results are identical
+ * to on = 0 (plain stream order).  CTR_EINVAL
  * for values other than 0 and 1.  No allocation; ctr_plan_get_launch_overlap returns it. */
 ctr_status ctr_plan_set_launch_overlap(ctr_plan *plan, int on);
 int ctr_plan_get_launch_overlap(const ctr_plan *plan);

@@ -17,7 +17,7 @@ ROOT = os.path.dirname(HERE)
 HEADERS = [os.path.join(ROOT, "include", "ctrecon.h"), os.path.join(SRC, "ctr_internal.cuh")]
 # kernels.cu includes radon.cu (which includes orbit.cuh and orbit64.cuh) and fft.cu: one translation unit, see its header
 INCLUDED = {"kernels.cu": ["radon.cu", "fft.cu", "orbit.cuh", "orbit64.cuh"]}
-UNITS = ["kernels.cu", "solver.cu", "capi.cu", "peak.cu"]
+UNITS = ["kernels.cu", "gfft.cu", "solver.cu", "capi.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -1111,7 +1111,7 @@ int ctr_plan_get_launch_overlap(const ctr_plan *p) { return p ? p->pdl : -1; }
 int ctr_plan_get_fft_form(const ctr_plan *p)
 {
     if (!p) return -1;
-    return (p->fft_form == 0 && wfft_supported(p)) ? 0 : 1;
+    return (p->fft_form == 0 && (wfft_supported(p) || (p->dtype != CTR_F64 && gfft_supported(p->n)))) ? 0 : 1;
 }
 
 ctr_status ctr_plan_get_fwd_shape(const ctr_plan *p, int *jobs_per_cta, int *segments)

@@ -445,7 +445,7 @@ struct ctr_plan {
     void *t1 = nullptr;        // N*M
     void *ubar_u = nullptr;    // n*n bar u of Alg. 5 (non-negativity)
     int pdl = 1;               // programmatic dependent launch of the iteration's kernels
-    int fft_form = 0;          // preconditioner passes: 0 warp-level where n allows (FP32, n = 256/512/1024), 1 CTA-level
+    int fft_form = 0;          // preconditioner passes: 0 warp-level where n allows (FP32; wfft_supported, gfft_supported), 1 CTA-level
     int precond_kind = 0;      // 0: inverse norm (Sec. 4.3.1); 1: impulse response; 2: circulant; 3: Richardson
     void *pk_s = nullptr;      // n*n DFT (2-D for kind 1, 1-D of the flattened image for kind 2) of the
                                // symmetrised impulse response of R_h^* R_h (built on first use)
@@ -526,6 +526,11 @@ int ramp_length(int M, size_t esize);   // FFT length of the ramp filter, 2^a 3^
 template <typename T>
 ctr_status launch_ramp(ctr_plan *p, const T *g, T *y, __nv_bfloat16 *yh, double outscale, cudaStream_t s);
 size_t fft_smem_bytes(const ctr_plan *p, int which);
+// the preconditioner's three passes for FP32 images of L V pixels, one warp per transform (gfft.cu);
+// part: the symmetric path's partial planes, else in_real
+bool gfft_supported(int n);
+ctr_status launch_gfft(bool pdl, int n, const float *in_real, const float *part, int groups, const BackprojEpi<float> &epi,
+                       float2 *cb, const float *sym, const float2 *tw, float *out, int mode, float *dout, cudaStream_t s);
 
 int backproject_tile_rows();   // pixel rows of a backprojection tile (its width is 32)
 template <typename T> bool bp_deferred(const ctr_plan *p);

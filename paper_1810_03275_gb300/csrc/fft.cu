@@ -1271,7 +1271,7 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
     // would overwrite unread input rows if the input were cbuf itself.
     if (p->precond_kind != 2 && (bp_in || !in_is_cbuf)) {
         if constexpr (sizeof(T) == 4) {
-            const int V = p->fft_form == 0 ? wfft_v(p) : 0;
+                        const int V = p->fft_form == 0 ? wfft_v(p) : 0;
             if (V) {
                 p->launches += 2;
                 const bool pdl = p->pdl != 0;
@@ -1280,6 +1280,15 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
                 else launch_wfft_packed<32>(pdl, src, cb, sym, tw, out, mode, outT, dout, outh, outTh, s);
                 CTR_CHECK_LAUNCH("k_wfft_packed");
                 return CTR_OK;
+            }
+            // Two-stage transforms where they exist (faster at every size, gfft.cu): their loads and
+            // folds are 16 bytes wide, and the transposed image of the per-angle projector, whose
+            // columns one warp would write 8 bytes at a time, stays with the passes below.
+            if (p->fft_form == 0 && gfft_supported(n) && !outT && !outh && !outTh && (!src.part || src.orbit) &&
+                (src.part || (uintptr_t)src.in_real % 16 == 0)) {
+                p->launches += 2;
+                return launch_gfft(p->pdl != 0, n, src.in_real, src.part, src.groups, src.epi, cb, sym, tw, out, mode, dout,
+                                   s);
             }
         }
         const int prp = packed_rows_per_cta(p), pcw = packed_cols_per_cta(p);
