@@ -119,7 +119,7 @@ def traffic_record(call: str):
         with open(path) as fh:
             d = json.load(fh)
         rec = d.get(call)
-        if rec and rec.get("src_sha") == src_sha("paper_1810_03275_gb300/csrc/radon.cu"):
+        if rec and rec.get("src_sha") == src_sha("paper_1810_03275_gb300/csrc/radon.cu", "paper_1810_03275_gb300/csrc/orbit.cuh"):
             return rec.get("dram_bytes_per_call")
     except Exception:
         pass
@@ -555,7 +555,7 @@ def main():
     reps = 20
     kt = {}
     sym = plan.symmetric_jobs > 0
-    call_kernels = {"rh_adjoint": ["k_backproject_orbit", "k_bp_fold"] if sym else
+    call_kernels = {"rh_adjoint": ["k_orbit_sino", "k_backproject_orbit", "k_bp_fold"] if sym else
                     (["k_backproject", "k_bp_reduce"] if plan.bp_groups > 1 else ["k_backproject"]),
                     "rh_forward_t": ["k_orbit_image", "k_forward_orbit"] if sym else ["k_forward"]}
     for name, fn in (("rh_adjoint", lambda: plan.rh_adjoint(f, u)), ("rh_forward_t", lambda: plan.rh_forward_t(u, uT, g))):

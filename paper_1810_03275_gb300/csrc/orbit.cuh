@@ -99,8 +99,9 @@ k_orbit_sino(const S *__restrict__ g, int M, int n_jobs, int list1, int pitch, i
 // and 5 differences for 8 pixels, and 4 shared-memory bins, where an interpolation per pixel
 // takes 24 operations and 16 bins.  One R_h^* call, 500^2 / 725 views (pair jobs): 85.6 us with an
 // interpolation per pixel, 38.9 us; 2048^2 / 2048 views: 2280 us, 975 us
-// (the packed FP32 pipe bounds it: fma.f32x2 on three distinct register pairs issues every third
-// cycle, about 130 of the 141 cycles a warp and job take on a scheduler).
+// (951 us of it this kernel: shared-memory pipe 76 % of its peak, FMA pipe 70 %, issue 62 %, and
+// the packed fma.f32x2 on three distinct register pairs issues every third cycle: about 130 of
+// the 141 cycles a warp and job take on a scheduler).
 //
 // offsets e0 = (C + 3S)/2, e1 = (C + S)/2, e2 = (C - S)/2, e3 = (C - 3S)/2: pixel (1, 3 - k)
 // sits at +e_k and pixel (0, k) at -e_k.  Jobs with 3 S <= C ("flat") have 0 <= e_k < 1:
@@ -382,11 +383,12 @@ ObpArgs obp_args(const ctr_plan *p, const float *bar)
 // tested.  A chunk of bins is as wide as the slots cover, [kb, kb + nb), nb = floor(64 A) - 1;
 // at the end the slots' three sums are gathered per bin through shared memory, in a fixed order,
 // and all of a job's warps share the epilogue.  One R_h call, 512^2 / 720 views: 69.9 us with the
-// march per bin, 57.2 us; 2048^2 / 2048 views: 2240 us, 1530 us.  The L1 pipe bounds it: an 8-byte
-// load of 32 pixels at an unaligned offset takes 3 wavefronts, 12 a row and warp (48 of the 51
-// cycles that 256 samples of four angles take on an SM at 2048^2).  Tried and slower: float4
-// records (64 cycles), the rows staged in shared memory by cp.async (62: the copies cost as much as
-// the loads), 32 warps a SM at 64 registers, an L1 prefetch 12 to 32 rows ahead (no change).
+// march per bin, 54.8 us; 2048^2 / 2048 views: 2240 us, 1530 us (L1 pipe 69 % of its peak, L2 62 %,
+// FMA 59 %, 37 % of the warp slots at 80 registers; an 8-byte load of 32 pixels at an unaligned
+// offset takes up to 3 wavefronts; at 512^2 54, 47 and 45 %: load latency).  Tried and slower: float4
+// records (512^2 59.8 us when planes took 57.7), the rows staged in shared memory by cp.async (86:
+// the copies cost as much as the loads), 32 warps a SM at 64 registers, an L1 prefetch 12 to 32 rows
+// ahead (no change).
 // ---------------------------------------------------------------------------
 constexpr int OFW_JOBS = 2, OFW_SEGS = 2, OFW_THREADS = 32 * OFW_JOBS * OFW_SEGS;   // of the batched stage
 
