@@ -466,12 +466,12 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
                 v[t].a = __ldg(ub + off + 32 * t);
                 if constexpr (NC == 4) v[t].b = __ldg(ub2 + off + 32 * t);
             }
-            const float xf = (float)r;                // x, in 2^-32 bins
+            const float xf = (float)r * 2.3283064365386963e-10f;   // x in bins (2^-32 of r: X stays in the range of u)
 #pragma unroll
             for (int t = 0; t < STRIPS; ++t) {
                 S[t] = vadd(S[t], v[t]);
                 X[t] = vfma(xf, v[t], X[t]);
-                Pp[t] = vfma(__saturatef(fmaf(xf, 2.3283064365386963e-10f, phi[t])), v[t], Pp[t]);
+                Pp[t] = vfma(__saturatef(xf + phi[t]), v[t], Pp[t]);
             }
             const bool step = r >= bound;
             r += step ? BA32 : B32;
@@ -480,7 +480,7 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
         // max(-z, 0) = max(z, 0) - z, z = x + phi
 #pragma unroll
         for (int t = 0; t < STRIPS; ++t)
-            Nn[t] = vfma(-phi[t], S[t], vfma(-2.3283064365386963e-10f, X[t], Pp[t]));
+            Nn[t] = vsub(vfma(-phi[t], S[t], Pp[t]), X[t]);
     }
 #pragma unroll
     for (int t = 0; t < STRIPS; ++t) {
