@@ -371,9 +371,11 @@ ObpArgs obp_args(const ctr_plan *p, const float *bar)
 // = x(m) lies in [0, A) on every row, so pixel slot s (0 <= s < 64) stays within one step
 // A <= 1 of s A + K0 and meets three bins only: its centre c = ceil(s A) and the two beside
 // it.  With z = x + s A - c in (-1, 1) a pixel adds max(z, 0) u to bin c + 1, max(-z, 0) u to
-// bin c - 1 and the rest to bin c; the lane sums u, x u and max(z, 0) u, which give all three.
+// bin c - 1 and the rest to bin c; the lane sums u, max(z, 0) u and max(-z, 0) u.  Rounding x
+// and s A - c is monotone and alike for both signs, so neither weight is positive where the exact
+// one is 0: a bin that no pixel touches comes out as exactly 0 (metal traces rely on it).
 // Each pixel of a row is read once by one lane, and x(m) is the same for the whole warp: per
-// slot 3 multiply-adds per channel and one for the weight, per row one conversion.
+// slot 3 multiply-adds per channel and two for the weights, per row one conversion.
 // (Marching one bin per lane instead reads two pixels per row, half of the second ones for
 // nothing, and does 4 multiply-adds.)
 //
@@ -422,9 +424,9 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
     const int kb = bx * nb;
     if (kb >= a.M) return;                            // CTA-uniform
     const bool active = slot < nj;                    // warp-uniform
-    V S[STRIPS], X[STRIPS], Pp[STRIPS], Nn[STRIPS];   // sums of u, x u, max(z, 0) u; of max(-z, 0) u at the end
+    V S[STRIPS], Pp[STRIPS], Nn[STRIPS];              // sums of u, max(z, 0) u and max(-z, 0) u
 #pragma unroll
-    for (int t = 0; t < STRIPS; ++t) S[t] = X[t] = Nn[t] = Pp[t] = vzero((V *)nullptr);
+    for (int t = 0; t < STRIPS; ++t) S[t] = Nn[t] = Pp[t] = vzero((V *)nullptr);
     const AngleMarch am = a.jobs[active ? jb : j0].am;
     const long long A = am.A, B = am.B, K0 = (long long)(kb - 1) << 32;
     // rows on which a slot may lie in the image, rounded out: q0(m) stays within [-66, n + 3]
@@ -466,21 +468,17 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
                 v[t].a = __ldg(ub + off + 32 * t);
                 if constexpr (NC == 4) v[t].b = __ldg(ub2 + off + 32 * t);
             }
-            const float xf = (float)r * 2.3283064365386963e-10f;   // x in bins (2^-32 of r: X stays in the range of u)
+            const float xf = (float)r;                // x, in 2^-32 bins
 #pragma unroll
             for (int t = 0; t < STRIPS; ++t) {
                 S[t] = vadd(S[t], v[t]);
-                X[t] = vfma(xf, v[t], X[t]);
-                Pp[t] = vfma(__saturatef(xf + phi[t]), v[t], Pp[t]);
+                Pp[t] = vfma(__saturatef(fmaf(xf, 2.3283064365386963e-10f, phi[t])), v[t], Pp[t]);
+                Nn[t] = vfma(__saturatef(fmaf(xf, -2.3283064365386963e-10f, -phi[t])), v[t], Nn[t]);
             }
             const bool step = r >= bound;
             r += step ? BA32 : B32;
             off += step ? pitch - 1 : pitch;
         }
-        // max(-z, 0) = max(z, 0) - z, z = x + phi
-#pragma unroll
-        for (int t = 0; t < STRIPS; ++t)
-            Nn[t] = vsub(vfma(-phi[t], S[t], Pp[t]), X[t]);
     }
 #pragma unroll
     for (int t = 0; t < STRIPS; ++t) {
