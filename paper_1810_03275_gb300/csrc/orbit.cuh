@@ -135,7 +135,7 @@ struct ObpArgs {
 };
 
 struct ObpTables {
-    uint4 *pos;    // {low, high word of the centre of the tile's first block in 2^-31 bins, C, S in 2^-31 bins}
+    uint4 *pos;    // {low, high word of the centre of the tile's first block in 2^-31 bins, C, S in 2^-32 bins}
     float4 *e;     // e0 .. e3
     long long *row;   // first staged bin (element of the orbit layout; of the detector with ObpArgs::g)
     int *flat;     // number of flat jobs of the table block
@@ -146,8 +146,9 @@ __device__ __forceinline__ void obp_job(const float2 *__restrict__ row, uint4 tp
                                         Vec<NC> &A, Vec<NC> &L0, Vec<NC> &L3, Vec<NC> (&KR)[4], Vec<NC> (&KL)[4])
 {
     using V = Vec<NC>;
-    const unsigned long long P = (((unsigned long long)tp.y << 32) | tp.x) + (unsigned long long)it * tp.z +
-                                 (unsigned long long)jt * tp.w;
+    // it and jt are even: their halves times C and S count 2^-31 bins
+    const unsigned long long P = (((unsigned long long)tp.y << 32) | tp.x) + (unsigned long long)(it >> 1) * tp.z +
+                                 (unsigned long long)(jt >> 1) * tp.w;
     const int b = (int)(P >> 31);
     const float f = (float)((unsigned)P & 0x7FFFFFFFu) * 4.656612873077393e-10f;   // 2^-31
     const float fm = f - 1.f;
@@ -220,7 +221,9 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
                 const long long P = (long long)i0 * C + (long long)j0 * S + am.Op + ((C + 3 * S) >> 1);
                 const int first = (int)((P >> 32) - 2 + a.pad) & ~1;                // 16-byte aligned
                 const unsigned long long base = (unsigned long long)(P - ((long long)(first - a.pad) << 32)) >> 1;
-                tb.pos[tid] = make_uint4((unsigned)base, (unsigned)(base >> 32), (unsigned)(C >> 1), (unsigned)(S >> 1));
+                // (C = 2^32, S = 0 of the axis: one unit less, 15 units of 2^-31 bins over the tile; the first
+                // block keeps its bin)
+                tb.pos[tid] = make_uint4((unsigned)base, (unsigned)(base >> 32), (unsigned)min(C, 0xFFFFFFFFll), (unsigned)S);
                 const float c = (float)C * 2.3283064365386963e-10f, s = (float)S * 2.3283064365386963e-10f;   // 2^-32
                 const bool flat = 3 * S <= C;
                 // (e3 = 0 up to rounding either way: both forms of the job then agree)
