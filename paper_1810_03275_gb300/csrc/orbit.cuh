@@ -182,7 +182,31 @@ __device__ __forceinline__ void obp_job(const float2 *__restrict__ row, uint4 tp
     }
 }
 
-template <int NC, bool NAMED>
+// One pixel of R_h^* over the jobs [la, lb), channel v, from the two bins beside its coordinate in
+// each: where the block form gives a value that is not finite.  A block's pixels share four or six
+// bins and their differences, so that a NaN or an infinite bin, or differences that overflow, would
+// reach pixels that do not interpolate from it.
+template <int NC>
+__device__ __noinline__ float pixel_alone(const float *bar, const float *g, const OrbitJob *jobs, int M, int pitch, int pad,
+                                          int la, int lb, int v, int i, int j)
+{
+    float acc = 0.f;
+    for (int t = la; t < lb; ++t) {
+        const AngleMarch am = jobs[t].am;
+        const long long P = (long long)i * am.A + (long long)j * am.B + am.Op;
+        const int k = (int)(P >> 32), l = jobs[t].l[v];
+        if (l < 0) continue;
+        const float *row = g ? g + (size_t)l * M : bar + 2 * ((size_t)t * (NC / 2) + (NC == 4 ? v >> 1 : 0)) * pitch + 2 * pad + (v & 1);
+        const int step = g ? 1 : 2;
+        const float g0 = (unsigned)k < (unsigned)M ? row[(long long)step * k] : 0.f;
+        const float g1 = (unsigned)(k + 1) < (unsigned)M ? row[(long long)step * (k + 1)] : 0.f;
+        acc = interp(acc, make_stage(g0, g1), P, 32, 0.0);
+    }
+    return acc;
+}
+
+// ALONE: a plain backprojection; a solver's preconditioner spreads values that are not finite anyway.
+template <int NC, bool NAMED, bool ALONE = false>
 __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int bz)
 {
     using V = Vec<NC>;
@@ -334,14 +358,30 @@ __device__ __forceinline__ void obp_body(const ObpArgs &a, int bx, int by, int b
                 }
             }
         }
+        if constexpr (ALONE) {
+            V sum = px[0][0];                                              // (not finite if one of them is not)
+#pragma unroll
+            for (int e = 1; e < 8; ++e) sum = vadd(sum, px[e >> 2][e & 3]);
+            bool finite = true;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) finite = finite && isfinite(vget(sum, c));
+            if (finite) continue;
+#pragma unroll 1
+            for (int e = 0; e < 8 * NC; ++e) {
+                const int v = li * NC + (e >> 3), ii = i + ((e >> 2) & 1), jj = j + (e & 3);
+                if (ii < a.n && jj < a.n)
+                    pg[(size_t)v * nn + (v < 2 ? (size_t)ii * a.n + jj : (size_t)jj * a.n + ii)] =
+                        pixel_alone<NC>(a.bar, a.g, a.jobs, a.M, a.pitch, a.pad, la, lb, v, ii, jj);
+            }
+        }
     }
 }
 
-template <int NC>
+template <int NC, bool ALONE>
 __global__ void __launch_bounds__(OBP_THREADS, 5) k_backproject_orbit(ObpArgs a)
 {
     pdl_wait();
-    obp_body<NC, false>(a, blockIdx.x, blockIdx.y, blockIdx.z);
+    obp_body<NC, false, ALONE>(a, blockIdx.x, blockIdx.y, blockIdx.z);
     pdl_trigger();
 }
 

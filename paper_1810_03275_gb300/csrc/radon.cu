@@ -889,7 +889,8 @@ ctr_status bp_impl(const ctr_plan *p, const S *g, const BackprojEpi<T> &epi, cud
                 bar = (const float *)p->gbar;
             }
             p->launches++;
-            auto kern = p->pair_jobs ? k_backproject_orbit<2> : k_backproject_orbit<4>;
+            auto kern = p->pair_jobs ? (defer_reduce ? k_backproject_orbit<2, false> : k_backproject_orbit<2, true>)
+                                     : (defer_reduce ? k_backproject_orbit<4, false> : k_backproject_orbit<4, true>);
             ObpArgs args = obp_args(p, bar);
             if (direct) args.g = (const float *)g;
             launch_pdl(p->pdl != 0, kern, grid, dim3(OBP_THREADS), obp_smem(p->pair_jobs ? 2 : 4), s,
@@ -988,8 +989,11 @@ ctr_status configure_radon(const ctr_plan *p)
     const size_t smem = bp_smem<T>(p);
     ctr_status st = raise_smem_limit(k_backproject<T, T>, smem);
     if (st == CTR_OK && p->orbit)
-        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2>, obp_smem(2), true)
-                          : raise_smem_limit(k_backproject_orbit<4>, obp_smem(4), true);
+        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2, false>, obp_smem(2), true)
+                          : raise_smem_limit(k_backproject_orbit<4, false>, obp_smem(4), true);
+    if (st == CTR_OK && p->orbit)
+        st = p->pair_jobs ? raise_smem_limit(k_backproject_orbit<2, true>, obp_smem(2), true)
+                          : raise_smem_limit(k_backproject_orbit<4, true>, obp_smem(4), true);
     if constexpr (sizeof(T) == 4)
         if (st == CTR_OK) st = raise_smem_limit(k_backproject<float, __nv_bfloat16>, smem);
     return st;

@@ -47,3 +47,27 @@ def test_forward(n, N, M, ds, dtype, value):
     must = (k == np.floor(p + SLACK)) & (k == np.floor(p - SLACK))
     may = (k >= np.floor(p - SLACK)) & (k <= np.floor(p + SLACK) + 1)
     _check(got, want, must, may, BOUND[dtype])
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "f64"])
+@pytest.mark.parametrize("n,N,M,ds", GEOMS)
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_adjoint(n, N, M, ds, dtype, value):
+    from paper_1810_03275_gb300 import ctrecon as ct
+    plan = ct.Plan(n, N, M, ds=ds, dtype=dtype)
+    assert plan.symmetric_jobs > 0 or dtype == "f64"      # (counts FP32 and BF16 jobs)
+    theta = np.arange(N) * (np.pi / N)
+    g = to_np(to_dev(np.random.default_rng(n).standard_normal((N, M)), plan.op_dtype))
+    spots = [(0, M // 2), (N // 6, M // 2 + 7), (N - 3, M // 2 - 9)]      # flat and steep views
+    for l, k in spots:
+        g[l, k] = 0.0
+    want = oracle.rh_adjoint(g, oracle.Geometry(n, N, M, ds=ds))
+    must = np.zeros((n, n), dtype=bool)
+    may = must.copy()
+    p = _coords(n, theta, M, ds)
+    for l, k in spots:
+        g[l, k] = value
+        must |= np.abs(p[l] - k) < 1 - SLACK
+        may |= np.abs(p[l] - k) < 1 + SLACK
+    got = to_np(plan.rh_adjoint(to_dev(g, plan.op_dtype)))
+    _check(got, want, must, may, BOUND[dtype])
