@@ -1344,75 +1344,42 @@ template ctr_status launch_fft2_forward<double>(const ctr_plan *, const double *
 // Detector-axis ramp filter (Sec. 2): per view, the bins zero-padded to L, forward FFT,
 // times the real multiplier H (the DFT of the Ram-Lak kernel wrapped onto L points, with
 // ds / L folded in), inverse FFT, the first M outputs times outscale: the linear
-// convolution of each view with the kernel.  H is real, so two views go through one complex
-// transform as its real and imaginary parts.  Rounding mixes the two, so that is done only
-// where their largest values are finite and within a factor of 64 of one another; else the
-// CTA transforms them one after the other.  1440 views of 1449 bins: 106 us with one view per
-// transform of 2916 points, 50 us with 3072.
+// convolution of each view with the kernel.  One view per transform and CTA: rounding in a transform
+// spreads over all that it holds, so a second view as the imaginary part, or the view's own even and
+// odd samples or two halves, would be cheaper and less exact (a smooth view, whose low frequencies
+// the filter removes: 4e-8 of it alone; with its samples split 2e-6, folded in the middle 9e-8;
+// beside a view 8 times as large 3e-5).  1440 views of 1449 bins: 81 us with transforms of 3072
+// points, 96 with 2916.
 template <typename T>
 __global__ void __launch_bounds__(FFT_THREADS)
-k_ramp_filter(const T *__restrict__ g, int N, int M, int L, FftPasses fp, const typename C2<T>::type *__restrict__ tw,
+k_ramp_filter(const T *__restrict__ g, int M, int L, FftPasses fp, const typename C2<T>::type *__restrict__ tw,
               const T *__restrict__ H, T outscale, T *y, __nv_bfloat16 *yh)
 {
     using T2 = typename C2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ T s_max[2][FFT_THREADS / 32];
     T2 *a = reinterpret_cast<T2 *>(smem_raw), *b = a + L, *stw = b + L;
     stage_twiddles(stw, tw, L);
-    const size_t r0 = (size_t)blockIdx.x * 2 * M;                        // the pair's views
-    const bool two = 2 * blockIdx.x + 1 < N;
-    T m0 = T(0), m1 = T(0);
-    bool finite = true;
+    const size_t r0 = (size_t)blockIdx.x * M;
+    for (int k = threadIdx.x; k < L; k += FFT_THREADS) {
+        T2 v;
+        v.x = k < M ? g[r0 + k] : T(0);
+        v.y = T(0);
+        a[k] = v;
+    }
+    twiddles_ready();
+    __syncthreads();
+    T2 *res = fft_smem<T>(a, b, L, 1, L, fp, -1, stw);
+    for (int k = threadIdx.x; k < L; k += FFT_THREADS) {
+        const T m = H[k];
+        res[k].x *= m;
+        res[k].y *= m;
+    }
+    __syncthreads();
+    T2 *res2 = fft_smem<T>(res, res == a ? b : a, L, 1, L, fp, +1, stw);
     for (int k = threadIdx.x; k < M; k += FFT_THREADS) {
-        const T v0 = g[r0 + k], v1 = two ? g[r0 + M + k] : T(0);
-        finite = finite && isfinite(v0) && isfinite(v1);
-        m0 = fmax(m0, v0 < T(0) ? -v0 : v0);
-        m1 = fmax(m1, v1 < T(0) ? -v1 : v1);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        m0 = fmax(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-        m1 = fmax(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_max[0][threadIdx.x >> 5] = m0;
-        s_max[1][threadIdx.x >> 5] = m1;
-    }
-    const bool all_finite = __syncthreads_and(finite) != 0;
-    for (int w = 0; w < FFT_THREADS / 32; ++w) {
-        m0 = fmax(m0, s_max[0][w]);
-        m1 = fmax(m1, s_max[1][w]);
-    }
-    const bool together = two && all_finite && m0 <= T(64) * m1 && m1 <= T(64) * m0;
-    const int turns = two && !together ? 2 : 1;
-    for (int t = 0; t < turns; ++t) {
-        if (t > 0) __syncthreads();
-        for (int k = threadIdx.x; k < L; k += FFT_THREADS) {
-            T2 v;
-            v.x = k < M ? g[r0 + (size_t)t * M + k] : T(0);
-            v.y = together && k < M ? g[r0 + M + k] : T(0);
-            a[k] = v;
-        }
-        twiddles_ready();
-        __syncthreads();
-        T2 *res = fft_smem<T>(a, b, L, 1, L, fp, -1, stw);
-        for (int k = threadIdx.x; k < L; k += FFT_THREADS) {
-            const T m = H[k];
-            res[k].x *= m;
-            res[k].y *= m;
-        }
-        __syncthreads();
-        T2 *res2 = fft_smem<T>(res, res == a ? b : a, L, 1, L, fp, +1, stw);
-        for (int k = threadIdx.x; k < M; k += FFT_THREADS) {
-            const T2 v = res2[k];
-            const size_t o = r0 + (size_t)t * M + k;
-            if (yh) {
-                yh[o] = __float2bfloat16_rn((float)(v.x * outscale));
-                if (together) yh[o + M] = __float2bfloat16_rn((float)(v.y * outscale));
-            } else {
-                y[o] = v.x * outscale;
-                if (together) y[o + M] = v.y * outscale;
-            }
-        }
+        const T v = res2[k].x * outscale;
+        if (yh) yh[r0 + k] = __float2bfloat16_rn((float)v);
+        else y[r0 + k] = v;
     }
 }
 
@@ -1463,8 +1430,8 @@ ctr_status launch_ramp(ctr_plan *p, const T *g, T *y, __nv_bfloat16 *yh, double 
     for (int i = 0; i < fp.count && i < MAX_PASSES; ++i) fp.radix[i] = p->ramp_radices[i];
     const int L = p->ramp_L;
     p->launches++;
-    k_ramp_filter<T><<<(p->N + 1) / 2, FFT_THREADS, ramp_smem(L, sizeof(T)), s>>>(
-        g, p->N, p->M, L, fp, reinterpret_cast<const typename C2<T>::type *>(p->d_ramp_tw),
+    k_ramp_filter<T><<<p->N, FFT_THREADS, ramp_smem(L, sizeof(T)), s>>>(
+        g, p->M, L, fp, reinterpret_cast<const typename C2<T>::type *>(p->d_ramp_tw),
         (const T *)p->d_ramp_H, (T)outscale, y, yh);
     CTR_CHECK_LAUNCH("k_ramp_filter");
     return CTR_OK;
