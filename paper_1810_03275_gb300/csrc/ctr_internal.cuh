@@ -52,6 +52,10 @@ struct NvtxScope {
 // completed and its writes are visible (and, since that kernel did the same, every
 // earlier one).  pdl_trigger() lets the next such launch be scheduled as soon as every CTA
 // of this grid is resident, so the launch latency overlaps the tail of this kernel.
+// What the kernel ahead writes is not read-only for the lifetime of a kernel launched so, nor is
+// what an earlier phase of the persistent batched kernel writes: such operands are read by
+// ordinary loads, through pointers that are not __restrict__ (__ldg and the read-only path are for
+// a plan's constants).
 // Both are no-ops for a kernel launched without the attribute.  The projectors trigger at
 // their CTAs' ends: triggered at their start, the next kernel's CTAs settle on the SMs that
 // run dry first and stay unevenly spread (Alg. 4, 384^2: 77 us an iteration against 72, 432^2:
@@ -152,7 +156,7 @@ struct BackprojEpi {
 // div_h p at pixel (i, j): (d1 + d2)/h, backward differences with Dirichlet ends
 // (Sec. 3.1); px holds the x plane, px + n*n the y plane.
 template <typename T>
-__device__ __forceinline__ T div_at(const T *__restrict__ px, int n, int i, int j, T inv_h)
+__device__ __forceinline__ T div_at(const T *px, int n, int i, int j, T inv_h)
 {
     if (n < 2) return T(0);
     const T *py = px + (size_t)n * n;
@@ -185,7 +189,7 @@ __device__ __forceinline__ T bp_epilogue_value(const BackprojEpi<T> &epi, int n,
 // The fold of the symmetric backprojection (OrbitJob path): its partial planes
 // [group][v][row][col] summed at image pixel (i, j) in a fixed order.
 template <typename T>
-__device__ __forceinline__ T orbit_fold(const T *__restrict__ part, int groups, int n, int i, int j)
+__device__ __forceinline__ T orbit_fold(const T *part, int groups, int n, int i, int j)
 {
     const size_t nn = (size_t)n * n;
     const size_t e = (size_t)i * n + j, em = (size_t)(n - 1 - i) * n + j;
@@ -205,7 +209,7 @@ __device__ __forceinline__ int pix_j(size_t e, int n) { return (int)((unsigned)e
 
 // The same fold for the four adjacent pixels (i, col .. col + 3) (col and n multiples of 4)
 // with 16-byte loads; each pixel's sum in the order of orbit_fold.
-__device__ __forceinline__ float4 orbit_fold4(const float *__restrict__ part, int groups, int n, int i, int col)
+__device__ __forceinline__ float4 orbit_fold4(const float *part, int groups, int n, int i, int col)
 {
     const size_t nn = (size_t)n * n;
     const size_t e = (size_t)i * n + col, em = (size_t)(n - 1 - i) * n + col;
@@ -213,10 +217,10 @@ __device__ __forceinline__ float4 orbit_fold4(const float *__restrict__ part, in
 #pragma unroll 4
     for (int z = 0; z < groups; ++z) {
         const float *pz = part + (size_t)z * 4 * nn;
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(pz + e));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(pz + nn + em));
-        const float4 c = __ldg(reinterpret_cast<const float4 *>(pz + 2 * nn + e));
-        const float4 d = __ldg(reinterpret_cast<const float4 *>(pz + 3 * nn + em));
+        const float4 a = *reinterpret_cast<const float4 *>(pz + e);
+        const float4 b = *reinterpret_cast<const float4 *>(pz + nn + em);
+        const float4 c = *reinterpret_cast<const float4 *>(pz + 2 * nn + e);
+        const float4 d = *reinterpret_cast<const float4 *>(pz + 3 * nn + em);
         s.x += a.x + b.x + c.x + d.x;
         s.y += a.y + b.y + c.y + d.y;
         s.z += a.z + b.z + c.z + d.z;
@@ -227,7 +231,7 @@ __device__ __forceinline__ float4 orbit_fold4(const float *__restrict__ part, in
 
 // grad_h u at pixel (i, j): forward differences with Neumann boundary (Sec. 3.1)
 template <typename T>
-__device__ __forceinline__ void grad_at(const T *__restrict__ u, int n, int i, int j, T inv_h, T &gx, T &gy)
+__device__ __forceinline__ void grad_at(const T *u, int n, int i, int j, T inv_h, T &gx, T &gy)
 {
     const size_t e = (size_t)i * n + j;
     const T c = u[e];

@@ -563,7 +563,7 @@ k_fft_cols_packed(typename C2<T>::type *cbuf, const T *__restrict__ sym, int n, 
 // epilogue as fft_rows_inv_body (the final values staged in the spare buffer for the
 // transposed writes).
 template <typename T>
-__device__ __forceinline__ void fft_rows_inv_packed_body(const typename C2<T>::type *__restrict__ cbuf, int n,
+__device__ __forceinline__ void fft_rows_inv_packed_body(const typename C2<T>::type *cbuf, int n,
                                                          int rows_per_cta, const FftPasses &fp,
                                                          const typename C2<T>::type *__restrict__ tw, T *out,
                                                          int mode, T *outT, T *dout, __nv_bfloat16 *outh,
@@ -631,7 +631,7 @@ __device__ __forceinline__ void fft_rows_inv_packed_body(const typename C2<T>::t
 
 template <typename T>
 __global__ void __launch_bounds__(FFT_THREADS)
-k_fft_rows_inv_packed(const typename C2<T>::type *__restrict__ cbuf, int n, int rows_per_cta, FftPasses fp,
+k_fft_rows_inv_packed(const typename C2<T>::type *cbuf, int n, int rows_per_cta, FftPasses fp,
                       const typename C2<T>::type *__restrict__ tw, T *out, int mode, T *outT, T *dout,
                       __nv_bfloat16 *outh, __nv_bfloat16 *outTh)
 {
@@ -642,7 +642,7 @@ k_fft_rows_inv_packed(const typename C2<T>::type *__restrict__ cbuf, int n, int 
 //   mode 0: out = v;  mode 1: out += v.   dout (optional) = v; outT (optional) =
 //   transpose of the final out.
 template <typename T>
-__device__ __forceinline__ void fft_rows_inv_body(const typename C2<T>::type *__restrict__ cbuf, int n,
+__device__ __forceinline__ void fft_rows_inv_body(const typename C2<T>::type *cbuf, int n,
                                                   int rows_per_cta, const FftPasses &fp,
                                                   const typename C2<T>::type *__restrict__ tw, T *out, int mode,
                                                   T *outT, T *dout, __nv_bfloat16 *outh, __nv_bfloat16 *outTh,
@@ -1022,7 +1022,7 @@ k_wfft_cols_packed(float2 *cbuf, const float *__restrict__ sym, const float2 *__
 // transposed copies written as (row 2c, row 2c + 1) pairs).
 template <int V>
 __global__ void __launch_bounds__(32 * WFFT_INV_WARPS)
-k_wfft_rows_inv_packed(const float2 *__restrict__ cbuf, const float2 *__restrict__ tw, float *out, int mode,
+k_wfft_rows_inv_packed(const float2 *cbuf, const float2 *__restrict__ tw, float *out, int mode,
                        float *outT, float *dout, __nv_bfloat16 *outh, __nv_bfloat16 *outTh)
 {
     constexpr int n = 32 * V, H = n / 2 + 1, G = 32 / V;

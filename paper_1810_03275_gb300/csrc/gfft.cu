@@ -172,7 +172,7 @@ constexpr int ROWS_THREADS = 256, COL_WARPS = 4, INV_WARPS = 2;
 // z = x_a + i x_b and writes X_a(k), X_b(k), k <= n / 2.
 template <int L, int V>
 __global__ void __launch_bounds__(ROWS_THREADS)
-k_gfft_rows_fwd(const float *__restrict__ in_real, const float *__restrict__ part, int groups, BackprojEpi<float> epi,
+k_gfft_rows_fwd(const float *in_real, const float *part, int groups, BackprojEpi<float> epi,
                 float2 *cbuf, const float2 *__restrict__ tw)
 {
     using T = Two<L, V>;
@@ -263,7 +263,7 @@ k_gfft_cols(float2 *cbuf, const float *__restrict__ sym, const float2 *__restric
 // -> row 2c + 1 (mode 0: out = v; mode 1: out += v; dout = v).
 template <int L, int V>
 __global__ void __launch_bounds__(32 * INV_WARPS)
-k_gfft_rows_inv(const float2 *__restrict__ cbuf, const float2 *__restrict__ tw, float *out, int mode, float *dout)
+k_gfft_rows_inv(const float2 *cbuf, const float2 *__restrict__ tw, float *out, int mode, float *dout)
 {
     using T = Two<L, V>;
     constexpr int n = T::n, H = T::H;

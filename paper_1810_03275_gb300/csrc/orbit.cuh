@@ -63,7 +63,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 // ---------------------------------------------------------------------------
 template <typename S, int NC>
 __global__ void __launch_bounds__(256)
-k_orbit_sino(const S *__restrict__ g, int M, int n_jobs, int list1, int pitch, int pad,
+k_orbit_sino(const S *g, int M, int n_jobs, int list1, int pitch, int pad,
              const OrbitJob *__restrict__ jobs, float *__restrict__ bar)
 {
     pdl_wait();
@@ -536,8 +536,8 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
             V v[STRIPS];
 #pragma unroll
             for (int t = 0; t < STRIPS; ++t) {
-                v[t].a = __ldg(ub + off + 32 * t);
-                if constexpr (NC == 4) v[t].b = __ldg(ub2 + off + 32 * t);
+                v[t].a = ub[off + 32 * t];
+                if constexpr (NC == 4) v[t].b = ub2[off + 32 * t];
             }
             const float xf = (float)r;                // x, in 2^-32 bins
 #pragma unroll

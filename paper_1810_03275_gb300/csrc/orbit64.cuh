@@ -32,7 +32,7 @@ struct Sym64Args {
 
 template <int NC>
 __global__ void __launch_bounds__(S64_THREADS)
-k_backproject_sym64(const double *__restrict__ g, Sym64Args a, double *__restrict__ part)
+k_backproject_sym64(const double *g, Sym64Args a, double *__restrict__ part)
 {
     __shared__ double2 s_bin[S64_JCH][NC][S64_WIN];
     __shared__ long long s_P[S64_JCH], s_C[S64_JCH], s_S[S64_JCH];
@@ -115,7 +115,7 @@ constexpr int F64_LANES = 32, F64_PAD = F64_LANES + 8, F64_SEGS = 4;
 constexpr int f64_pitch(int n) { return n + 2 * F64_PAD; }
 
 __global__ void __launch_bounds__(256)
-k_orbit_image64(const double *__restrict__ u, double *__restrict__ ubar, int n)
+k_orbit_image64(const double *u, double *ubar, int n)
 {
     __shared__ double tC[32][33], tD[32][33];
     pdl_wait();
@@ -151,7 +151,7 @@ __device__ __forceinline__ double pos64(double z)
 // preconditioner spreads such values anyway, and 64^2 / 90 views lose 5 % of an iteration to it)
 template <int NC, bool ALONE>
 __global__ void __launch_bounds__(32 * F64_SEGS)
-k_forward_sym64(const double *__restrict__ ubar, Sym64Args a, ForwardEpi<double> epi)
+k_forward_sym64(const double *ubar, Sym64Args a, ForwardEpi<double> epi)
 {
     constexpr int LN = F64_LANES, NT = 32 * F64_SEGS;
     __shared__ double s_part[F64_SEGS][NC][3 * LN];   // the slots' sums for bins c, c + 1, c - 1
@@ -194,7 +194,7 @@ k_forward_sym64(const double *__restrict__ ubar, Sym64Args a, ForwardEpi<double>
             double v[NC];
 #pragma unroll
             for (int h = 0; h < NC / 2; ++h) {
-                const double2 w = __ldg(ub + h * plane + off);
+                const double2 w = ub[h * plane + off];
                 v[2 * h] = w.x;
                 v[2 * h + 1] = w.y;
             }

@@ -135,9 +135,9 @@ __device__ __forceinline__ void bp_epilogue(const BackprojEpi<T> &epi, int n, in
 // part == nullptr: apply the epilogue directly (one angle group).  Otherwise write
 // this group's partial sums to part[bz][n][n].
 template <typename T, typename S, bool NAMED = false>
-__device__ __forceinline__ void bp_body(const S *__restrict__ g, int n, int N, int M, int F, int wstride,
+__device__ __forceinline__ void bp_body(const S *g, int n, int N, int M, int F, int wstride,
                                         int angles_per_group, const AngleGeom *__restrict__ geom,
-                                        const BackprojEpi<T> &epi, T *__restrict__ part, int bx, int by, int bz)
+                                        const BackprojEpi<T> &epi, T *part, int bx, int by, int bz)
 {
     using T2 = typename Pair<T>::type;
     constexpr int NT = 32 * BP_TY;
@@ -346,7 +346,7 @@ __device__ __forceinline__ void forward_epilogue_pre(const ForwardEpi<float> &ep
 // One row of the march: the NC candidate pixels q, q+1, ... of the lane's interval.
 // EXACT1: the first candidate is always inside the interval (A <= 2^F, i.e. h <= ds).
 template <typename T, typename S, int NC, bool EXACT1>
-__device__ __forceinline__ void march_row(const S *__restrict__ rowp, int dq, int n, int k, int F, double inv2F,
+__device__ __forceinline__ void march_row(const S *rowp, int dq, int n, int k, int F, double inv2F,
                                           long long Pa, int q, long long A, T &Su, T &Sf)
 {
     {
@@ -378,7 +378,7 @@ constexpr int FWD_THREADS = 32 * FWD_AW;
 // q_a back when r >= thr = A - B, B <= 0 steps it forward when r < thr = |B|.
 // CHECK = false: every lane's q_a and q_a + 1 are inside [0, n) on these rows.
 template <int DQ, bool BPOS, bool CHECK, typename S>
-__device__ __forceinline__ void march32(const S *__restrict__ base, int n, int rows, unsigned &r, int &q, int &off,
+__device__ __forceinline__ void march32(const S *base, int n, int rows, unsigned &r, int &q, int &off,
                                         unsigned A32, unsigned lim, unsigned B32, unsigned thr, float &Su, float &Sf)
 {
 #pragma unroll FWD_UNROLL
@@ -411,7 +411,7 @@ __device__ __forceinline__ void march32(const S *__restrict__ base, int n, int r
 // The FP32 march of one lane over rows [mlo, mhi] of the warp, without bounds checks on
 // the warp's interior rows [ilo, ihi] (mlo <= ilo, ihi <= mhi; ilo > ihi: none).
 template <int DQ, bool BPOS, typename S>
-__device__ __forceinline__ void march32_rows(const S *__restrict__ base, int n, long long K, const AngleMarch &am,
+__device__ __forceinline__ void march32_rows(const S *base, int n, long long K, const AngleMarch &am,
                                              int mlo, int mhi, int ilo, int ihi, float &Su, float &Sf)
 {
     const long long A = am.A, B = am.B;
@@ -436,7 +436,7 @@ __device__ __forceinline__ void march32_rows(const S *__restrict__ base, int n, 
 // Sum u and sum frac u (FP64) or sum (1 + frac) u (generic FP32) over the pixels of rows
 // m0 .. m0 + rows - 1 whose detector coordinate lies in the lane's interval [k, k+1).
 template <typename T, typename S, int NC, bool EXACT1>
-__device__ __forceinline__ void fwd_march(const S *__restrict__ base, int dq, int n, int k, int F,
+__device__ __forceinline__ void fwd_march(const S *base, int dq, int n, int k, int F,
                                           const AngleMarch &am, int m0, int rows, T &Su, T &Sf)
 {
     const double inv2F = ldexp(1.0, -F);
@@ -495,7 +495,7 @@ __device__ __forceinline__ void rows_in(float Q0, float binv, float qlo, float q
 // bx*31 + [0, 31).  The angles are adjacent, so their rays nearly coincide and the
 // image rows they read are shared in L1.
 template <typename T, typename S, int NC, bool EXACT1>
-__device__ __forceinline__ void fwd_body(const S *__restrict__ u, const S *__restrict__ uT, int n, int N, int M, int F,
+__device__ __forceinline__ void fwd_body(const S *u, const S *uT, int n, int N, int M, int F,
                                          const AngleMarch *__restrict__ march, const ForwardEpi<T> &epi, int bx, int by)
 {
     const int warp = threadIdx.x >> 5;
@@ -506,7 +506,7 @@ __device__ __forceinline__ void fwd_body(const S *__restrict__ u, const S *__res
     if (l >= N || kb >= M) return;                    // warp-uniform
     const AngleMarch am = march[l];
     // pixel (m, q) of the march is at base[m*n + dq*q]
-    const S *__restrict__ base = (am.layout ? u : uT) + (am.flip ? (n - 1) : 0);
+    const S *base = (am.layout ? u : uT) + (am.flip ? (n - 1) : 0);
     // q*(m) = Q0 - m b: the real pick coordinate where P(q, m) = k 2^F
     const float Q0 = (float)k * am.kA - am.oA;
     int mlo, mhi;                                     // rows where the lane's pixel run may be inside [0, n)
@@ -558,7 +558,7 @@ k_forward(const S *__restrict__ u, const S *__restrict__ uT, int n, int N, int M
 // FP32 (a BF16 plan's operand is widened here).  Rows of
 // orbit_pitch pixels, pixel 0 at ORBIT_PAD; the pads keep the zeros they got when the plan was
 // made.  Two planes (float2): channels {0, 1}, then {2, 3}.
-__device__ __forceinline__ void orbit_store(float *__restrict__ ubar, size_t plane, size_t o, float a, float b, float c,
+__device__ __forceinline__ void orbit_store(float *ubar, size_t plane, size_t o, float a, float b, float c,
                                             float d)
 {
     reinterpret_cast<float2 *>(ubar)[o] = make_float2(a, b);
@@ -568,7 +568,7 @@ __device__ __forceinline__ void orbit_store(float *__restrict__ ubar, size_t pla
 // 32 x 32 tiles: four coalesced tile loads (two of them transposed through shared
 // memory), one coalesced record store per pixel.
 template <typename S>
-__device__ __forceinline__ void orbit_image_body(const S *__restrict__ u, float *__restrict__ ubar, int n, int bx, int by)
+__device__ __forceinline__ void orbit_image_body(const S *u, float *ubar, int n, int bx, int by)
 {
     __shared__ float tA[32][33], tB[32][33], tC[32][33], tD[32][33];
     const size_t pitch = orbit_pitch(n), plane = pitch * n;
@@ -597,7 +597,7 @@ __device__ __forceinline__ void orbit_image_body(const S *__restrict__ u, float 
 
 template <typename S>
 __global__ void __launch_bounds__(256)
-k_orbit_image(const S *__restrict__ u, float *__restrict__ ubar, int n)
+k_orbit_image(const S *u, float *ubar, int n)
 {
     pdl_wait();
     pdl_trigger();
@@ -610,7 +610,7 @@ k_orbit_image(const S *__restrict__ u, float *__restrict__ ubar, int n)
 // its forward neighbours comes from tile A (rows m, columns q, plus a one-pixel halo), so
 // the kernel waits on global memory once; the arithmetic is that of tv_dual_at.
 __global__ void __launch_bounds__(256)
-k_orbit_image_tv(const float *__restrict__ u, float *__restrict__ ubar, int n, TvDualJob<float> tv)
+k_orbit_image_tv(const float *u, float *ubar, int n, TvDualJob<float> tv)
 {
     pdl_wait();
     pdl_trigger();
@@ -740,7 +740,7 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c)
 // backprojection epilogue (grid-stride over the pixels).
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_bp_fold(const T *__restrict__ part, int groups, int n, BackprojEpi<T> epi)
+k_bp_fold(const T *part, int groups, int n, BackprojEpi<T> epi)
 {
     pdl_wait();
     pdl_trigger();

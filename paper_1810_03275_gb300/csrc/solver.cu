@@ -115,7 +115,7 @@ __global__ void k_init_y2(const T *__restrict__ u, const T *__restrict__ v2b, in
 // Step D of Alg. 4: TV dual update with the projection onto the ball of radius lam/tau.
 // ub (Alg. 5 only): bar u += max(2 u - bar u, 0) - u, the resolvent of I_{u >= 0}.
 template <typename T>
-__device__ __forceinline__ void tv_dual_body(const T *__restrict__ u, int n, T sigma, T tau, T lam, T inv_h, T *v2b,
+__device__ __forceinline__ void tv_dual_body(const T *u, int n, T sigma, T tau, T lam, T inv_h, T *v2b,
                                              T *y2, T *t2, T *ub, int b, int nb)
 {
     const size_t nn = (size_t)n * n;
@@ -126,7 +126,7 @@ __device__ __forceinline__ void tv_dual_body(const T *__restrict__ u, int n, T s
 
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_tv_dual(const T *__restrict__ u, int n, T sigma, T tau, T lam, T inv_h, T *v2b, T *y2, T *t2, T *ub)
+k_tv_dual(const T *u, int n, T sigma, T tau, T lam, T inv_h, T *v2b, T *y2, T *t2, T *ub)
 {
     pdl_wait();
     pdl_trigger();
@@ -251,7 +251,7 @@ __device__ __forceinline__ T block_uniform(F f)
 
 // x = y / sqrt(scal[idx])   (scal holds a squared norm)
 template <typename T>
-__global__ void k_normalize(const T *__restrict__ y, size_t len, const double *__restrict__ scal, int idx, T *x)
+__global__ void k_normalize(const T *y, size_t len, const double *scal, int idx, T *x)
 {
     pdl_wait();
     pdl_trigger();
@@ -292,7 +292,7 @@ __device__ __forceinline__ void block_reduce(double (&v)[NV], unsigned maxmask, 
 }
 
 template <int NV>
-__global__ void __launch_bounds__(RED_THREADS) k_finalize(const double *__restrict__ part, int nblk, unsigned maxmask, double *out)
+__global__ void __launch_bounds__(RED_THREADS) k_finalize(const double *part, int nblk, unsigned maxmask, double *out)
 {
     pdl_wait();
     pdl_trigger();
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_finalize(const double *__restri
 
 // (sum a*b, sum b*b)
 template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) k_dot2(const T *__restrict__ a, const T *__restrict__ b, size_t len, double *part)
+__global__ void __launch_bounds__(RED_THREADS) k_dot2(const T *a, const T *b, size_t len, double *part)
 {
     pdl_wait();
     pdl_trigger();
