@@ -652,7 +652,7 @@ k_forward_orbit(OfwArgs a, ForwardEpi<float> epi)
 {
     pdl_wait();
     // chunks from the detector's middle outwards: the long rays first, the short ones fill the tail
-    const int c = blockIdx.y, mid = (gridDim.y - 1) / 2;
+    const int c = blockIdx.z * gridDim.y + blockIdx.y, mid = (gridDim.y * gridDim.z - 1) / 2;
     ofw_body<NC, JOBS, SEGS, false, ALONE>(a, epi, c & 1 ? mid + (c + 1) / 2 : mid - c / 2, blockIdx.x);
     pdl_trigger();
 }
@@ -666,7 +666,10 @@ int ofw_groups(const ctr_plan *p, int jobs)
 template <int JOBS, int SEGS>
 void launch_forward_orbit_shape(const ctr_plan *p, const float *ub, const ForwardEpi<float> &epi, cudaStream_t s)
 {
-    const dim3 grid(ofw_groups(p, JOBS), p->fwd_chunks);
+    // (chunks beyond a grid's 65535 rows, detectors of some millions of bins, go on in z; what is
+    // left over there lies beyond the detector)
+    const int z = (p->fwd_chunks + 65534) / 65535;
+    const dim3 grid(ofw_groups(p, JOBS), (p->fwd_chunks + z - 1) / z, z);
     auto kern = p->pair_jobs
                     ? (epi.mode == 0 ? k_forward_orbit<2, JOBS, SEGS, true> : k_forward_orbit<2, JOBS, SEGS, false>)
                     : (epi.mode == 0 ? k_forward_orbit<4, JOBS, SEGS, true> : k_forward_orbit<4, JOBS, SEGS, false>);
