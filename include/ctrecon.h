@@ -355,14 +355,13 @@ ctr_status ctr_plan_set_bp_groups(ctr_plan *plan, int groups);
 int ctr_plan_get_bp_groups(const ctr_plan *plan);
 
 /* Tuning hook: the launch shape of the symmetric forward projector, one of the compiled
- * instances (jobs_per_cta, segments) = (1, 2), (1, 4) [default], (1, 8), (2, 2), (2, 4),
- * (4, 2), (4, 1).  A CTA takes jobs_per_cta adjacent jobs (nearly coincident rays: they
+ * instances (jobs_per_cta, segments) = (1, 2), (1, 4), (1, 8), (2, 2), (2, 4), (4, 2), (4, 1).  A CTA takes jobs_per_cta adjacent jobs (nearly coincident rays: they
  * share the orbit image's lines in L1) and a chunk of bins; `segments` warps split the rows each
- * job's rays cross, and their sums are added in a fixed order.  The default (1, 4) leaves the
- * choice to the library, which takes (2, 4) or (2, 2) where there is enough work.  The shape
- * changes FP32 summation order only.  CTR_EINVAL for other shapes, CTR_EUNSUPPORTED off the
+ * job's rays cross, and their sums are added in a fixed order.  Until one is set the library
+ * chooses: (1, 4), or (2, 4) or (2, 2) where there is enough work.  The shape changes FP32
+ * summation order only.  CTR_EINVAL for other shapes, CTR_EUNSUPPORTED off the
  * symmetric path and, for (4, 1), where the rays of four adjacent jobs are far apart;
- * ctr_plan_get_fwd_shape reports the shape set, and (0, 0) off the symmetric path. */
+ * ctr_plan_get_fwd_shape reports the shape that is launched, and (0, 0) off the symmetric path. */
 ctr_status ctr_plan_set_fwd_shape(ctr_plan *plan, int jobs_per_cta, int segments);
 ctr_status ctr_plan_get_fwd_shape(const ctr_plan *plan, int *jobs_per_cta, int *segments);
 

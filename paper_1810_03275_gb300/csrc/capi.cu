@@ -1117,8 +1117,8 @@ int ctr_plan_get_fft_form(const ctr_plan *p)
 ctr_status ctr_plan_get_fwd_shape(const ctr_plan *p, int *jobs_per_cta, int *segments)
 {
     if (!p || !jobs_per_cta || !segments) return fail(CTR_EINVAL, "null argument");
-    *jobs_per_cta = p->orbit ? p->fwd_slots : 0;
-    *segments = p->orbit ? p->fwd_segs : 0;
+    *jobs_per_cta = p->orbit ? fwd_shape(p) / 16 : 0;
+    *segments = p->orbit ? fwd_shape(p) % 16 : 0;
     return CTR_OK;
 }
 

@@ -473,8 +473,8 @@ struct ctr_plan {
     int red_blocks = 0;
     cudaStream_t stream = nullptr;       // internal stream (graph capture)
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-    int fwd_slots = 1;                   // symmetric forward projector: adjacent jobs per CTA (1, 2, 4) ...
-    int fwd_segs = 4;                    // ... and warps splitting a job's rows (2, 4, 8); see ctr_plan_set_fwd_shape
+    int fwd_slots = 0;                   // symmetric forward projector, as set: adjacent jobs per CTA (1, 2, 4) ...
+    int fwd_segs = 0;                    // ... and warps splitting a job's rows (1, 2, 4, 8); 0: see fwd_shape
     bool shape41 = false;                // ctr_plan_set_fwd_shape takes (4, 1)
     double *d_hist = nullptr;            // MAX_CHECKS x HIST_FIELDS diagnostics records
     int hist_count = 0;                  // records the last solve wrote
@@ -542,6 +542,7 @@ template <typename T> bool bp_deferred(const ctr_plan *p);
 // orbit image): callers may then skip making the transposed copy uT
 template <typename T> inline bool fwd_needs_transpose(const ctr_plan *p) { return !(sizeof(T) == 4 && p->orbit) && !p->sym64; }
 int fwd_grid_x(int M);         // forward-projector grid: bin chunks
+int fwd_shape(const ctr_plan *p);               // its launch shape, jobs * 16 + segments, set or the library's choice
 int ofw_batch_groups(const ctr_plan *p);        // symmetric forward projector, batched stage: groups of jobs
 int orbit_fwd_chunks(const std::vector<OrbitJob> &jobs, int M, int F);
 size_t sym64_image_bytes(int n);     // orbit image of an FP64 plan   // symmetric forward projector: bin chunks per job

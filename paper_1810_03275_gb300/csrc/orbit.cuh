@@ -676,19 +676,18 @@ void launch_forward_orbit_shape(const ctr_plan *p, const float *ub, const Forwar
     launch_pdl(p->pdl != 0, kern, grid, dim3(32 * JOBS * SEGS), 0, s, OfwArgs{ub, p->d_jobs, p->n, p->M, p->n_jobs, p->job_list[1]}, epi);
 }
 
-// The launch shape (jobs * 16 + segments): the one ctr_plan_set_fwd_shape chose, or for its default
-// (1, 4) the one measured best for the number of (job, chunk) pairs there are: with many, two
+// The launch shape (jobs * 16 + segments): the one ctr_plan_set_fwd_shape set, else the one
+// measured best for the number of (job, chunk) pairs there are: with many, two
 // adjacent jobs share their image lines in L1 (four-channel jobs 2048^2: (2, 4) 1530 us, (1, 4)
 // 1740; 512^2 with 3077 pairs: 57 either way.  Pair jobs 2048^2 / 2047 views: (2, 2) 1813, (1, 4) 1879;
 // 500^2 / 725 with 6171 pairs: 61.6 and 62.4); with few, splitting rows over four warps matters more
 // (256^2: (1, 4) 17.8, (2, 2) 24.1).
 int ofw_shape(const ctr_plan *p)
 {
-    const int shape = p->fwd_slots * 16 + p->fwd_segs;
-    if (shape != 1 * 16 + 4) return shape;
+    if (p->fwd_slots > 0) return p->fwd_slots * 16 + p->fwd_segs;
     const long long pairs = (long long)p->n_jobs * p->fwd_chunks;
-    if (p->pair_jobs) return pairs >= 8000 ? 2 * 16 + 2 : shape;
-    return pairs >= 4000 ? 2 * 16 + 4 : shape;
+    if (p->pair_jobs) return pairs >= 8000 ? 2 * 16 + 2 : 1 * 16 + 4;
+    return pairs >= 4000 ? 2 * 16 + 4 : 1 * 16 + 4;
 }
 
 void launch_forward_orbit(const ctr_plan *p, const float *ub, const ForwardEpi<float> &epi, cudaStream_t s)

@@ -1047,6 +1047,8 @@ template bool bp_deferred<double>(const ctr_plan *);
 
 int fwd_grid_x(int M) { return (M + 30) / 31; }
 
+int fwd_shape(const ctr_plan *p) { return ofw_shape(p); }
+
 int ofw_batch_groups(const ctr_plan *p) { return ofw_groups(p, OFW_JOBS); }
 
 size_t sym64_image_bytes(int n) { return 2 * sizeof(double2) * (size_t)n * f64_pitch(n); }

@@ -565,8 +565,7 @@ inline void plan_state_key(const ctr_plan *p, std::vector<double> &k)
     k.push_back((double)p->obp_groups);
     k.push_back((double)p->precond_kind);
     k.push_back((double)p->alg3);
-    k.push_back((double)p->fwd_slots);
-    k.push_back((double)p->fwd_segs);
+    k.push_back((double)fwd_shape(p));
     k.push_back((double)p->fft_form);
     k.push_back((double)p->pdl);
 }
