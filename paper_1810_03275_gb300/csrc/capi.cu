@@ -689,6 +689,12 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
         destroy(p);
         return fail(CTR_ECUDA, "stream/event creation failed");
     }
+    // the tables' copies and the pads' zeroing were put on the default stream, which streams that do
+    // not synchronise with it would overtake
+    if (cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        destroy(p);
+        return fail(CTR_ECUDA, "plan tables: copy failed");
+    }
     *out = p;
     return CTR_OK;
 }

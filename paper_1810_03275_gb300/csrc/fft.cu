@@ -1414,6 +1414,7 @@ ctr_status prepare_ramp(ctr_plan *p)
     }
     CTR_CUDA(cudaMemcpy(p->d_ramp_tw, tw.data(), sizeof(T) * tw.size(), cudaMemcpyHostToDevice));
     CTR_CUDA(cudaMemcpy(p->d_ramp_H, H.data(), sizeof(T) * H.size(), cudaMemcpyHostToDevice));
+    CTR_CUDA(cudaStreamSynchronize(cudaStreamLegacy));                 // (the caller's stream may not wait for them)
     ctr_status st = raise_smem_limit(k_ramp_filter<T>, ramp_smem(L, sizeof(T)));
     if (st != CTR_OK) return st;
     p->ramp_ready = true;

@@ -1761,6 +1761,7 @@ ctr_status batch_prepare(ctr_batch *b)
     }
     for (int stg = 0; stg < BS_COUNT; ++stg) b->blocks[stg] = pre[(size_t)stg * (ns + 1) + ns];
     CTR_CUDA(cudaMemcpy(b->d_prefix, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice));
+    CTR_CUDA(cudaStreamSynchronize(cudaStreamLegacy));             // (a solve's stream may not wait for it)
     ctr_status st = configure_batch_radon(b->smem[BS_BP], b->smem[BS_BP_SYM]);
     if (st == CTR_OK) st = configure_batch_fft(b->smem[BS_FFT_ROWS], b->smem[BS_FFT_COLS]);
     if (st != CTR_OK) return st;
