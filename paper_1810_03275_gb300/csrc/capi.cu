@@ -671,13 +671,14 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
         int cap = p->bp_groups;
         if (p->n <= 1024) cap = maxg < MAX_BP_GROUPS ? (maxg > cap ? maxg : cap) : MAX_BP_GROUPS;
         p->bp_cap = cap;
-        if (cap > 1) ALLOC(p->bp_part, es * nn * cap);
     }
     ALLOC(p->d_red, sizeof(double) * 8 * p->red_blocks);
     ALLOC(p->d_scal, sizeof(double) * 64);
     ALLOC(p->d_hist, sizeof(double) * HIST_FIELDS * MAX_CHECKS);
-#undef ALLOC
     if ((st = build_tables(p)) != CTR_OK) { destroy(p); return st; }
+    // the partial images (the FP64 symmetric path has its own partial planes there)
+    if (p->bp_cap > 1 && !p->sym64) ALLOC(p->bp_part, es * nn * p->bp_cap);
+#undef ALLOC
     st = (dtype == CTR_F64) ? build_twiddles<double>(p) : build_twiddles<float>(p);
     if (st != CTR_OK) { destroy(p); return st; }
     st = (dtype == CTR_F64) ? configure_radon<double>(p) : configure_radon<float>(p);
