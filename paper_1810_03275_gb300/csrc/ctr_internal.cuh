@@ -561,9 +561,10 @@ template <typename T> ctr_status launch_orbit_bar(const ctr_plan *p, const T *g,
 void bp_tiles(int n, int &tx, int &ty);
 int fft_rows_per_cta(int n);
 bool wfft_supported(const ctr_plan *p);        // the warp-level preconditioner passes apply
-int fft_packed_rows_per_cta(const ctr_plan *p); // real-input form of the CTA-level passes: row pairs x 2 per CTA
-int fft_packed_cols_per_cta(const ctr_plan *p); // ... stored columns per CTA
-size_t fft_packed_smem(const ctr_plan *p, int which);   // ... dynamic shared memory (0 rows, 1 columns)
+// the real-input form of the CTA-level passes, `images` of them in one launch:
+int fft_packed_rows_per_cta(const ctr_plan *p, int images);        // row pairs x 2 per CTA
+int fft_packed_cols_per_cta(const ctr_plan *p, int images);        // stored columns per CTA
+size_t fft_packed_smem(const ctr_plan *p, int images, int which);  // dynamic shared memory (0 rows, 1 columns)
 size_t fft_rows_smem(int n, size_t esize);   // dynamic shared memory of the row passes
 size_t fft_cols_smem(int n, size_t esize);   // ... and of the column pass
 int fft_cols_per_cta(int n, size_t esize);

@@ -65,7 +65,7 @@ constexpr int MAX_PASSES = 16;
 #ifndef CTR_FFT_MIN_CTAS
 #define CTR_FFT_MIN_CTAS 128
 #endif
-constexpr int FFT_MIN_CTAS = CTR_FFT_MIN_CTAS;   // CTAs a real-input pass is split into, where it has as many transforms
+constexpr int FFT_MIN_CTAS = CTR_FFT_MIN_CTAS;   // CTAs a real-input pass over all images is split into, where it has as many transforms
 
 
 template <typename T> struct C2;
@@ -1214,27 +1214,40 @@ int cols_per_cta(const ctr_plan *p) { return fft_cols_per_cta(p->n, p->esize); }
 #endif
 // (a small image is spread over as many CTAs as it has transforms: the passes are bound by the
 // latency of one CTA's chain, in FP64 by its SM's two FP64 lanes.  FP64 64^2 with the fold, the
-// column pass and the inverse: 32, 15.5 and 10.5 us on 4, 9 and 4 CTAs)
-int packed_rows_per_cta(const ctr_plan *p)
+// column pass and the inverse: 32, 15.5 and 10.5 us on 4, 9 and 4 CTAs.  A batch fills the chip with
+// its images together, and more CTAs than that would only idle their threads: split for 128 CTAs
+// each, an iteration of 64 images of 64^2 takes 101 us, of 128^2 351, of 256^2 940; split for 128 in
+// all 63, 261 and 826.)
+int share(int images) { return std::max(1, FFT_MIN_CTAS / images); }
+int packed_rows_per_cta(const ctr_plan *p, int images)
 {
     const int pairs = fft_rows_per_cta(p->n) > 1 ? fft_rows_per_cta(p->n) / 2 : 1;
-    return 2 * CTR_PACK_ROWS_MUL * std::max(1, std::min(pairs, p->n / 2 / FFT_MIN_CTAS));
+    return 2 * CTR_PACK_ROWS_MUL * std::max(1, std::min(pairs, p->n / 2 / share(images)));
 }
-int packed_cols_per_cta(const ctr_plan *p)
+int packed_cols_per_cta(const ctr_plan *p, int images)
 {
     int c = CTR_PACK_COLS_MUL * (cols_per_cta(p) > 1 ? cols_per_cta(p) / 2 : 1);
     while (c > 1 && 2 * (size_t)c * (p->n + 1) * 2 * p->esize > 160 * 1024) c /= 2;
-    return std::max(1, std::min(c, (p->n / 2 + 1) / FFT_MIN_CTAS));
+    return std::max(1, std::min(c, (p->n / 2 + 1) / share(images)));
 }
-size_t packed_rows_smem(const ctr_plan *p) { return (2 * (size_t)(packed_rows_per_cta(p) / 2) * p->n + p->n) * 2 * p->esize; }
-size_t packed_cols_smem(const ctr_plan *p) { return (2 * (size_t)packed_cols_per_cta(p) * (p->n + 1) + p->n) * 2 * p->esize; }
+size_t packed_rows_smem(const ctr_plan *p, int images)
+{
+    return (2 * (size_t)(packed_rows_per_cta(p, images) / 2) * p->n + p->n) * 2 * p->esize;
+}
+size_t packed_cols_smem(const ctr_plan *p, int images)
+{
+    return (2 * (size_t)packed_cols_per_cta(p, images) * (p->n + 1) + p->n) * 2 * p->esize;
+}
 
 }  // namespace
 
 bool wfft_supported(const ctr_plan *p) { return wfft_v(p) != 0; }
-int fft_packed_rows_per_cta(const ctr_plan *p) { return packed_rows_per_cta(p); }
-int fft_packed_cols_per_cta(const ctr_plan *p) { return packed_cols_per_cta(p); }
-size_t fft_packed_smem(const ctr_plan *p, int which) { return which == 0 ? packed_rows_smem(p) : packed_cols_smem(p); }
+int fft_packed_rows_per_cta(const ctr_plan *p, int images) { return packed_rows_per_cta(p, images); }
+int fft_packed_cols_per_cta(const ctr_plan *p, int images) { return packed_cols_per_cta(p, images); }
+size_t fft_packed_smem(const ctr_plan *p, int images, int which)
+{
+    return which == 0 ? packed_rows_smem(p, images) : packed_cols_smem(p, images);
+}
 
 size_t fft_smem_bytes(const ctr_plan *p, int which)
 {
@@ -1291,9 +1304,9 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
                                    s);
             }
         }
-        const int prp = packed_rows_per_cta(p), pcw = packed_cols_per_cta(p);
+        const int prp = packed_rows_per_cta(p, 1), pcw = packed_cols_per_cta(p, 1);
         const int pgr = (n + prp - 1) / prp, pgc = (n / 2 + 1 + pcw - 1) / pcw;
-        const size_t psr = packed_rows_smem(p), psc = packed_cols_smem(p);
+        const size_t psr = packed_rows_smem(p, 1), psc = packed_cols_smem(p, 1);
         const bool pdl = p->pdl != 0 && pgr <= 304;    // (more CTAs crowd on the SMs that run dry first: 768^2 264 us against 246)
         launch_pdl(pdl, k_fft_rows_fwd_packed<T>, dim3(pgr), dim3(FFT_THREADS), psr, s, src, cb, n, prp, fp, tw);
         CTR_CHECK_LAUNCH("k_fft_rows_fwd_packed");
@@ -1447,9 +1460,9 @@ ctr_status configure_fft(const ctr_plan *p)
     ctr_status st = raise_smem_limit(k_fft_rows_fwd<T>, smr);
     if (st == CTR_OK) st = raise_smem_limit(k_fft_rows_inv<T>, smr);
     if (st == CTR_OK) st = raise_smem_limit(k_fft_cols<T>, smc);
-    if (st == CTR_OK) st = raise_smem_limit(k_fft_rows_fwd_packed<T>, packed_rows_smem(p));
-    if (st == CTR_OK) st = raise_smem_limit(k_fft_rows_inv_packed<T>, packed_rows_smem(p));
-    if (st == CTR_OK) st = raise_smem_limit(k_fft_cols_packed<T>, packed_cols_smem(p));
+    if (st == CTR_OK) st = raise_smem_limit(k_fft_rows_fwd_packed<T>, packed_rows_smem(p, 1));
+    if (st == CTR_OK) st = raise_smem_limit(k_fft_rows_inv_packed<T>, packed_rows_smem(p, 1));
+    if (st == CTR_OK) st = raise_smem_limit(k_fft_cols_packed<T>, packed_cols_smem(p, 1));
     return st;
 }
 

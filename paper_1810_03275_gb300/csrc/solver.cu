@@ -1605,8 +1605,8 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.rpc = fft_rows_per_cta(p->n);
         d.cw = fft_cols_per_cta(p->n, 4);
         d.packed = batch_slice_packed(b, p);
-        d.prp = fft_packed_rows_per_cta(p);
-        d.pcw = fft_packed_cols_per_cta(p);
+        d.prp = fft_packed_rows_per_cta(p, ns);
+        d.pcw = fft_packed_cols_per_cta(p, ns);
         d.geom = p->d_geom;
         d.march = p->d_march;
         d.cbuf = (float2 *)p->cbuf;
@@ -1736,8 +1736,8 @@ ctr_status batch_prepare(ctr_batch *b)
         bp_tiles(p->n, tx, ty);
         const size_t nn = (size_t)p->n * p->n;
         const bool packed = batch_slice_packed(b, p);
-        const int rpc = packed ? fft_packed_rows_per_cta(p) : fft_rows_per_cta(p->n);
-        const int cw = fft_cols_per_cta(p->n, 4), pcw = fft_packed_cols_per_cta(p);
+        const int rpc = packed ? fft_packed_rows_per_cta(p, ns) : fft_rows_per_cta(p->n);
+        const int cw = fft_cols_per_cta(p->n, 4), pcw = fft_packed_cols_per_cta(p, ns);
         int cnt[BS_COUNT];
         const int t32 = (p->n + 31) / 32;
         cnt[BS_BP] = p->orbit ? 0 : tx * ty * p->bp_groups;
@@ -1752,8 +1752,8 @@ ctr_status batch_prepare(ctr_batch *b)
         for (int stg = 0; stg < BS_COUNT; ++stg) pre[(size_t)stg * (ns + 1) + i + 1] = pre[(size_t)stg * (ns + 1) + i] + cnt[stg];
         const size_t smb = p->orbit ? 0 : bp_smem_bytes(p->wstride), smo = p->orbit ? obp_smem_bytes(p) : 0;
         if (smo > b->smem[BS_BP_SYM]) b->smem[BS_BP_SYM] = smo;
-        const size_t smr = packed ? fft_packed_smem(p, 0) : fft_rows_smem(p->n, sizeof(float));
-        const size_t smc = packed ? fft_packed_smem(p, 1) : fft_cols_smem(p->n, sizeof(float));
+        const size_t smr = packed ? fft_packed_smem(p, ns, 0) : fft_rows_smem(p->n, sizeof(float));
+        const size_t smc = packed ? fft_packed_smem(p, ns, 1) : fft_cols_smem(p->n, sizeof(float));
         if (smb > b->smem[BS_BP]) b->smem[BS_BP] = smb;
         if (smr > b->smem[BS_FFT_ROWS]) b->smem[BS_FFT_ROWS] = smr;
         if (smr > b->smem[BS_FFT_ROWS_INV]) b->smem[BS_FFT_ROWS_INV] = smr;
