@@ -599,10 +599,13 @@ ctr_status ctr_plan_create(const ctr_geometry *g, ctr_dtype dtype, ctr_plan **ou
     ctr_status st = fft_radices(p->n, p->radices);
     p->fft_ok = (st == CTR_OK);
     if (!p->fft_ok) p->radices.clear();
-    if (dtype == CTR_F64 && p->n < 1024) {
+    if (dtype == CTR_F64 && p->n < 256) {
         // FP64: a warp instruction takes 64 cycles of its scheduler however many lanes work, so
         // a pass is as long as its butterfly and radix 2 keeps the most lanes busy (64^2: a
-        // radix-8 pass has 8 butterflies of about 100 operations, a radix-2 one 32 of 10)
+        // radix-8 pass has 8 butterflies of about 100 operations, a radix-2 one 32 of 10).  From
+        // 256^2 up larger radices fill the lanes too, and have fewer barriers.  M^{-1} y, us, radix 2
+        // against mixed: 64^2 24.4 and 28.8, 96^2 24.4 and 26.3, 128^2 24.7 and 31.6, 192^2 29.6 and
+        // 33.9, 256^2 39.5 and 37.2, 384^2 59.5 and 58.4, 512^2 82.4 and 67.1, 768^2 138 and 118
         std::vector<int> small;
         for (int r : p->radices)
             if (r == 3) small.push_back(3);
