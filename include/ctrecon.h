@@ -165,14 +165,18 @@ unsigned long long ctr_plan_launch_count(const ctr_plan *plan);
  * two angles or more on average, the unpaired angle 0 of an odd count aside (uniform angles
  * over [0, pi): an even count in jobs of up to four angles, an odd count in (N + 1) / 2 jobs
  * of theta and pi - theta, which the FP32 kernels run as two-channel "pair" jobs).
- * Results equal those of the per-angle path up to the order of FP32 summation. */
+ * Results equal those of the per-angle path up to FP32 rounding.  (FP64 plans take a symmetric path
+ * too, which this count does not report.) */
 int ctr_plan_symmetric_jobs(const ctr_plan *plan);
 
 /* g = R_h u, the discrete Radon transform of Sec. 3.1 (the adjoint of linear
  * backprojection): bin k of angle l gets sum_ij u_ij Lambda(p_ijl - k) with
  * p = (x_i cos theta_l + y_j sin theta_l)/ds + (M-1)/2 and the hat
  * Lambda(t) = max(0, 1 - |t|).  u_dev: n*n, g_dev: N*M (overwritten).
- * Ray-driven gather (no atomics); exact transpose of rh_adjoint. */
+ * Ray-driven gather (no atomics); the transpose of rh_adjoint (angle by angle and in FP64 the same
+ * weights, on the symmetric path in FP32 up to their rounding).  A bin that no pixel reaches is
+ * exactly 0; a pixel that is not finite reaches the bins on either side of its p in each view and
+ * no others. */
 ctr_status rh_forward(ctr_plan *plan, const void *u_dev, void *g_dev, void *stream);
 
 /* rh_forward for a caller that also holds the transposed image uT_dev[j*n + i] =
@@ -182,7 +186,9 @@ ctr_status rh_forward_t(ctr_plan *plan, const void *u_dev, const void *uT_dev, v
 
 /* u = R_h^* g, linear backprojection (Sec. 3.1, definition of R_h^*): pixel (i,j)
  * gets sum_l of g linearly interpolated at p_ijl.  g_dev: N*M, u_dev: n*n
- * (overwritten).  Pixel-driven gather. */
+ * (overwritten).  Pixel-driven gather.  On the symmetric path in FP32 weights hold to 2^-22 bins,
+ * and a bin leaves up to 2^-22 of its value in pixels within a few bins of it that do not
+ * interpolate from it; a bin that is not finite reaches the pixels within one bin of it only. */
 ctr_status rh_adjoint(ctr_plan *plan, const void *g_dev, void *u_dev, void *stream);
 
 /* x = M^{-1} y, the inverse-norm Fourier preconditioner of Alg. 4 (Sec. 4.3.1, 4.4):
@@ -231,7 +237,7 @@ ctr_status tv_pd_solve(ctr_plan *plan, const void *f_dev, const uint8_t *metal_m
  * N*M in the plan's real type (float for FP32 and BF16 plans).  The filter tables are
  * built on the first call (synchronous), later calls are asynchronous on `stream`.
  * CTR_EUNSUPPORTED when one padded view does not fit a CTA's shared memory (FP64 plans
- * with more than about 1600 bins, FP32 beyond about 4600). */
+ * with more than 2304 bins, FP32 beyond 4608). */
 ctr_status ctr_ramp_filter(ctr_plan *plan, const void *g_dev, void *y_dev, void *stream);
 
 /* Filtered backprojection u = (pi / N) R_h^*(ramp-filtered g) (Sec. 2, uniform angles over

@@ -132,13 +132,9 @@ ctr_status build_sym64(ctr_plan *p, const std::vector<OrbitJob> &jobs)
     return CTR_OK;
 }
 
-// Groups the angles of a plan into the forward projector's symmetric jobs
-// (OrbitJob): every angle's (C, S) must be one of (a, b), (-a, b), (b, a), (-b, a) of
-// its canonical pair a = max(|C|, |S|), b = min(|C|, |S|) (true for angles in
-// [0, pi)); angles with equal canonical pairs share a job, one per channel.  The
-// path is taken when the jobs hold two angles or more on average.
 // Whether ctr_plan_set_fwd_shape takes (4, 1): two blocks of 8 rows of the pixels that four
-// consecutive jobs (in the order of their first angles) cross must fit one CTA's shared memory.
+// consecutive jobs (in the order of their first angles) cross must fit one CTA's shared memory.  The
+// shape's instance needs no such memory; the rule keeps refused what the interface refuses.
 bool shape41_fits(const std::vector<OrbitJob> &jobs, int n, int M)
 {
     const double one = 4294967296.0;
@@ -163,6 +159,11 @@ bool shape41_fits(const std::vector<OrbitJob> &jobs, int n, int M)
     return 2.0 * 8 * std::floor(w) * 16 + 2.0 * sizeof(int) * ((n + 8) / 8 + 1) <= 227 * 1024;
 }
 
+// Groups the angles of a plan into the forward projector's symmetric jobs
+// (OrbitJob): every angle's (C, S) must be one of (a, b), (-a, b), (b, a), (-b, a) of
+// its canonical pair a = max(|C|, |S|), b = min(|C|, |S|) (true for angles in
+// [0, pi)); angles with equal canonical pairs share a job, one per channel.  The
+// path is taken when the jobs hold two angles or more on average.
 ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
 {
     const int n = p->n, N = p->N, M = p->M, F = p->F;
@@ -270,10 +271,12 @@ ctr_status build_orbit_jobs(ctr_plan *p, const std::vector<AngleGeom> &geo)
     if ((st = alloc(p, &p->ubar, sizeof(float4) * (size_t)n * orbit_pitch(n))) != CTR_OK) return st;
     CTR_CUDA(cudaMemset(p->ubar, 0, sizeof(float4) * (size_t)n * orbit_pitch(n)));   // the pads stay zero
     p->fwd_chunks = orbit_fwd_chunks(jobs, M, F);
-    // the symmetric backprojection: job groups so that tiles x groups is about 1024 CTAs
-    // (~1.7 waves of 4 eight-warp CTAs per SM on 152 SMs; measured best at n = 512 among
-    // 2..8), at least 8 jobs per group; room for up to MAX_BP_GROUPS groups at n <= 1024
-    // so that ctr_plan_set_bp_groups can change the split later
+    // the symmetric backprojection: job groups so that tiles x groups is about 1024 CTAs of four
+    // warps (five fit an SM: 1.35 waves), at least 8 jobs per group.  R_h^*, us, by groups (chosen
+    // first): 512^2 / 720 views 4: 34.8, 3: 34.5, 2: 44.7, 8: 36.7; 256^2 / 360 8: 13.5, 4: 16.4;
+    // 432^2 / 600 5: 24.5, 4: 24.9, 8: 27.1; 432^2 / 361 (pair jobs) 5: 22.3, 3: 19.8, 2: 20.8;
+    // 500^2 / 725 4: 39.9, 5: 41.6; 1024^2 / 1440 1: 194, 2: 192, 4: 194.  Room for up to
+    // MAX_BP_GROUPS groups at n <= 1024 so that ctr_plan_set_bp_groups can change the split later
     const int tiles = ((n + 31) / 32) * ((n + 31) / 32);
     int G = (1024 + tiles / 2) / tiles;
     if (G > MAX_BP_GROUPS) G = MAX_BP_GROUPS;

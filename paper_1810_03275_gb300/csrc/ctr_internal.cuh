@@ -106,10 +106,12 @@ template <> struct Cplx<double> { using type = double2; };
 //     p = (x_i cos theta_l + y_j sin theta_l)/ds + (M-1)/2,
 // is represented exactly as the integer P = i*C + j*S + O in units of 2^-F bins,
 // with C = round(2^F h cos/ds), S = round(2^F h sin/ds) and O chosen so that the
-// grid is centred.  floor(p) = P >> F and frac(p) = (P mod 2^F) 2^-F.  Both
-// projectors derive every interpolation weight from the same integer P, so the
-// ray-driven R_h is the exact transpose of the pixel-driven R_h^*.
-// F = 32 for FP32/BF16 (weight = top 23 fraction bits), F = 51 or less for FP64 (48 at 4096^2).
+// grid is centred.  floor(p) = P >> F and frac(p) = (P mod 2^F) 2^-F.  F = 32 for
+// FP32/BF16, F = 51 or less for FP64 (48 at 4096^2).  Both projectors start from the same
+// integer P.  Angle by angle (weight = top 23 fraction bits in FP32) and in FP64 they form the
+// same weights from it, so that the ray-driven R_h is the exact transpose of the pixel-driven
+// R_h^*; the symmetric path's FP32 projectors round x + s A - c and f + o apart, each to FP32,
+// and are adjoint up to that rounding.
 // ---------------------------------------------------------------------------
 struct AngleGeom {
     long long C, S, O;
@@ -308,7 +310,7 @@ struct FftPasses {
 
 // One slice of a batch: everything a batched stage kernel needs (FP32).
 struct SliceDesc {
-    int n, N, M, wstride, bp_groups, per_group;
+    int n, N, M, wstride, bp_groups, per_group;   // per_group: views per group (per-angle path)
     int bp_tiles_x, bp_tiles_y;   // backprojection tiles
     int fwd_chunks;               // forward-projector CTAs per angle
     int rpc, cw;                  // FFT rows / columns per CTA
@@ -320,7 +322,7 @@ struct SliceDesc {
     const float *sym;
     FftPasses fp;
     float *u, *uT, *y1, *y2, *v2b, *bp_part;   // bp_part: angle-group images, or the symmetric planes
-    int orbit;                    // symmetric projector path (per_group, bp_groups count jobs)
+    int orbit;                    // symmetric projector path (bp_groups counts job groups)
     int pair_jobs;                // the symmetric projectors' pair-job variants
     int twist;                    // the circulant preconditioner's 1-D transform in the column pass
     float *ub;                    // Alg. 5: bar u (updated by the TV stage); null for Alg. 4

@@ -1284,7 +1284,7 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
     // would overwrite unread input rows if the input were cbuf itself.
     if (p->precond_kind != 2 && (bp_in || !in_is_cbuf)) {
         if constexpr (sizeof(T) == 4) {
-                        const int V = p->fft_form == 0 ? wfft_v(p) : 0;
+            const int V = p->fft_form == 0 ? wfft_v(p) : 0;
             if (V) {
                 p->launches += 2;
                 const bool pdl = p->pdl != 0;
@@ -1294,7 +1294,8 @@ ctr_status launch_circulant(const ctr_plan *p, const T *in_real, bool in_is_cbuf
                 CTR_CHECK_LAUNCH("k_wfft_packed");
                 return CTR_OK;
             }
-            // Two-stage transforms where they exist (faster at every size, gfft.cu): their loads and
+            // Two-stage transforms where they exist (faster up to 648^2 and in M^{-1} y alone, equal inside
+            // an iteration at 768^2 and 864^2: gfft.cu): their loads and
             // folds are 16 bytes wide, and the transposed image of the per-angle projector, whose
             // columns one warp would write 8 bytes at a time, stays with the passes below.
             if (p->fft_form == 0 && gfft_supported(n) && !outT && !outh && !outTh && (!src.part || src.orbit) &&

@@ -10,10 +10,11 @@
 // barrier after each of four or five stages and the same again for the inverse.  Here a transform
 // waits once each way, for its transposition through shared memory (rows padded to an odd length:
 // both directions are free of bank conflicts), and every butterfly is in registers.
-// An iteration of Alg. 4 (n / 2 views), CTA-level -> two-stage, us: 64^2 25.6 -> 19.4,
-// 128^2 30.4 -> 23.4, 216^2 38.2 -> 30.2, 384^2 54.3 -> 44.1, 432^2 60.8 -> 48.8,
-// 576^2 79.3 -> 73.1, 648^2 104 -> 91, 768^2 137.4 -> 137.3, 864^2 170 -> 169; M^{-1} y alone
-// 768^2 33.6 -> 23.0, 864^2 38.7 -> 33.5.  Error against 64 bits 1.9e-7 .. 2.8e-7 in both.
+// An iteration of Alg. 4 (n / 2 views), CTA-level -> two-stage, us: 64^2 24.6 -> 18.4,
+// 128^2 30.6 -> 23.8, 216^2 38.1 -> 30.1, 384^2 54.3 -> 44.2, 432^2 61.1 -> 48.8,
+// 576^2 79.8 -> 73.6, 648^2 103 -> 91, 768^2 136.9 -> 135.9, 864^2 172 -> 170 (there the projectors
+// hide it); M^{-1} y alone 768^2 33.1 -> 25 (launched by the host: 22 to 27), 864^2 37.4 -> 33.0.
+// Error against 64 bits 1.9e-7 .. 2.8e-7 in both.
 #include "ctr_internal.cuh"
 
 namespace ctr {

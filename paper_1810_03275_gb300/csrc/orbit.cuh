@@ -63,7 +63,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src)
 // ---------------------------------------------------------------------------
 template <typename S, int NC>
 __global__ void __launch_bounds__(256)
-k_orbit_sino(const S *g, int M, int n_jobs, int list1, int pitch, int pad,
+k_orbit_sino(const S *g, int M, int list1, int pitch, int pad,
              const OrbitJob *__restrict__ jobs, float *__restrict__ bar)
 {
     pdl_wait();
@@ -98,8 +98,8 @@ k_orbit_sino(const S *g, int M, int n_jobs, int list1, int pitch, int pad,
 // right knot, half only the left.  Per block, job and channel that is 12 fused multiply-adds
 // and 5 differences for 8 pixels, and 4 shared-memory bins, where an interpolation per pixel
 // takes 24 operations and 16 bins.  One R_h^* call, 500^2 / 725 views (pair jobs): 85.6 us with an
-// interpolation per pixel, 38.9 us; 2048^2 / 2048 views: 2280 us, 975 us
-// (951 us of it this kernel: shared-memory pipe 76 % of its peak, FMA pipe 70 %, issue 62 %, and
+// interpolation per pixel, 39.7 us; 2048^2 / 2048 views: 2280 us, 980 us
+// (951 of 975 us this kernel: shared-memory pipe 76 % of its peak, FMA pipe 70 %, issue 62 %, and
 // the packed fma.f32x2 on three distinct register pairs issues every third cycle: about 130 of
 // the 141 cycles a warp and job take on a scheduler).
 //
@@ -108,6 +108,10 @@ k_orbit_sino(const S *g, int M, int n_jobs, int list1, int pitch, int pad,
 // four bins b - 1 .. b + 2.  The others have e3 < 0 (those two pixels swap knots) and e0 up
 // to 1.42 (two more knots, bins b - 2 .. b + 3).  The jobs of a list are sorted by S / C, so
 // each chunk is a run of flat jobs and a run of steep ones.
+//
+// A pixel's terms of bins that it does not interpolate from cancel only up to rounding: a bin leaves
+// up to 2^-22 of its value (as much as a weight's own rounding) in the other pixels of the blocks
+// whose bins b - 2 .. b + 3 hold it.
 //
 // Bank conflicts: an 8-byte load is served sixteen lanes at a time; they hold 8 x 2 blocks,
 // whose bins span 14 C + 4 S <= 14.6 plus one: distinct or equal modulo sixteen.
@@ -455,9 +459,11 @@ __device__ __noinline__ T bin_alone(const T *pix, int pitch, int n, long long A,
 // tested.  A chunk of bins is as wide as the slots cover, [kb, kb + nb), nb = floor(64 A) - 1;
 // at the end the slots' three sums are gathered per bin through shared memory, in a fixed order,
 // and all of a job's warps share the epilogue.  One R_h call, 512^2 / 720 views: 69.9 us with the
-// march per bin, 54.8 us; 2048^2 / 2048 views: 2240 us, 1530 us (L1 pipe 69 % of its peak, L2 62 %,
+// march per bin, 56.1 us; 2048^2 / 2048 views: 2240 us, 1588 us (with max(-z, 0) u formed at the end from
+// u and x u, which left rounding in untouched bins: 54.8 and 1537; L1 pipe 69 % of its peak, L2 62 %,
 // FMA 59 %, 37 % of the warp slots at 80 registers; an 8-byte load of 32 pixels at an unaligned
-// offset takes up to 3 wavefronts; at 512^2 54, 47 and 45 %: load latency).  Tried and slower: float4
+// offset takes up to 3 wavefronts; at 512^2 54, 47 and 45 %: load latency; both before max(-z, 0) u
+// was summed by itself).  Tried and slower: float4
 // records (512^2 59.8 us when planes took 57.7), the rows staged in shared memory by cp.async (86:
 // the copies cost as much as the loads), 32 warps a SM at 64 registers, an L1 prefetch 12 to 32 rows
 // ahead (no change).
@@ -678,10 +684,10 @@ void launch_forward_orbit_shape(const ctr_plan *p, const float *ub, const Forwar
 
 // The launch shape (jobs * 16 + segments): the one ctr_plan_set_fwd_shape set, else the one
 // measured best for the number of (job, chunk) pairs there are: with many, two
-// adjacent jobs share their image lines in L1 (four-channel jobs 2048^2: (2, 4) 1530 us, (1, 4)
-// 1740; 512^2 with 3077 pairs: 57 either way.  Pair jobs 2048^2 / 2047 views: (2, 2) 1813, (1, 4) 1879;
-// 500^2 / 725 with 6171 pairs: 61.6 and 62.4); with few, splitting rows over four warps matters more
-// (256^2: (1, 4) 17.8, (2, 2) 24.1).
+// adjacent jobs share their image lines in L1 (four-channel jobs 2048^2: (2, 4) 1588 us, (1, 4)
+// 1798; 1024^2 / 1440: 309 and 336; 512^2 with 3077 pairs: 56 either way.  Pair jobs 2048^2 / 2047 views:
+// (2, 2) 1965, (1, 4) 2000; 500^2 / 725 with 6171 pairs: 62.1 and 61.4); with few, splitting rows over
+// four warps matters more (256^2: (1, 4) 17.5, (2, 2) 25.7).
 int ofw_shape(const ctr_plan *p)
 {
     if (p->fwd_slots > 0) return p->fwd_slots * 16 + p->fwd_segs;

@@ -19,7 +19,8 @@
 //    No atomics; each output bin is written once.
 // Both kernels derive each weight from the same integer P (see ctr_internal.cuh),
 // so they are transposes of one matrix.  Plans whose angles are symmetric images of
-// one another take the kernels of orbit.cuh instead, which use the same integers.
+// one another take the kernels of orbit.cuh (FP64: orbit64.cuh) instead, which start from the same
+// integers; in FP32 they round their weights apart, so that the pair is adjoint up to FP32 rounding.
 #include <algorithm>
 #include <type_traits>
 
@@ -865,7 +866,7 @@ ctr_status launch_orbit_sino(const ctr_plan *p, const S *g, float *bar, cudaStre
     p->launches++;
     const dim3 grid((p->M + 255) / 256, p->n_jobs);
     auto kern = p->pair_jobs ? k_orbit_sino<S, 2> : k_orbit_sino<S, 4>;
-    launch_pdl(p->pdl != 0, kern, grid, dim3(256), 0, s, g, p->M, p->n_jobs, p->job_list[1], p->bar_pitch, p->bar_pad,
+    launch_pdl(p->pdl != 0, kern, grid, dim3(256), 0, s, g, p->M, p->job_list[1], p->bar_pitch, p->bar_pad,
                (const OrbitJob *)p->d_jobs, bar);
     CTR_CHECK_LAUNCH("k_orbit_sino");
     return CTR_OK;

@@ -1598,8 +1598,7 @@ ctr_status batch_solve(ctr_batch *b, const float *const *f, const uint8_t *const
         d.obp_win = p->obp_win;
         for (int k = 0; k < 3; ++k) d.job_list[k] = p->job_list[k];
         d.bp_groups = p->orbit ? p->obp_groups : p->bp_groups;
-        d.per_group = p->orbit ? (p->n_jobs + p->obp_groups - 1) / p->obp_groups
-                               : (p->N + p->bp_groups - 1) / p->bp_groups;
+        d.per_group = (p->N + p->bp_groups - 1) / p->bp_groups;
         bp_tiles(p->n, d.bp_tiles_x, d.bp_tiles_y);
         d.fwd_chunks = p->orbit ? p->fwd_chunks : fwd_grid_x(p->M);
         d.rpc = fft_rows_per_cta(p->n);
