@@ -111,6 +111,10 @@ def src_sha(*rel):
     return h.hexdigest()[:16]
 
 
+#: the sources of the operators' kernels: a traffic record holds for exactly these
+OPERATOR_SOURCES = [f"paper_1810_03275_gb300/csrc/{f}" for f in ("radon.cu", "orbit.cuh", "ctr_internal.cuh")]
+
+
 def traffic_record(call: str):
     """DRAM bytes per operator call (summed over the kernels it launches) from the
     committed ncu summary, if it was taken on the current kernel source (else None)."""
@@ -119,7 +123,7 @@ def traffic_record(call: str):
         with open(path) as fh:
             d = json.load(fh)
         rec = d.get(call)
-        if rec and rec.get("src_sha") == src_sha("paper_1810_03275_gb300/csrc/radon.cu", "paper_1810_03275_gb300/csrc/orbit.cuh"):
+        if rec and rec.get("src_sha") == src_sha(*OPERATOR_SOURCES):
             return rec.get("dram_bytes_per_call")
     except Exception:
         pass

@@ -200,7 +200,8 @@ __device__ __noinline__ float pixel_alone(const float *bar, const float *g, cons
         const long long P = (long long)i * am.A + (long long)j * am.B + am.Op;
         const int k = (int)(P >> 32), l = jobs[t].l[v];
         if (l < 0) continue;
-        const float *row = g ? g + (size_t)l * M : bar + 2 * ((size_t)t * (NC / 2) + (NC == 4 ? v >> 1 : 0)) * pitch + 2 * pad + (v & 1);
+        const size_t plane = (size_t)t * (NC / 2) + (NC == 4 ? v >> 1 : 0);
+        const float *row = g ? g + (size_t)l * M : bar + 2 * (plane * pitch + pad) + (v & 1);
         const int step = g ? 1 : 2;
         const float g0 = (unsigned)k < (unsigned)M ? row[(long long)step * k] : 0.f;
         const float g1 = (unsigned)(k + 1) < (unsigned)M ? row[(long long)step * (k + 1)] : 0.f;
@@ -460,13 +461,12 @@ __device__ __noinline__ T bin_alone(const T *pix, int pitch, int n, long long A,
 // at the end the slots' three sums are gathered per bin through shared memory, in a fixed order,
 // and all of a job's warps share the epilogue.  One R_h call, 512^2 / 720 views: 69.9 us with the
 // march per bin, 56.1 us; 2048^2 / 2048 views: 2240 us, 1588 us (with max(-z, 0) u formed at the end from
-// u and x u, which left rounding in untouched bins: 54.8 and 1537; L1 pipe 69 % of its peak, L2 62 %,
-// FMA 59 %, 37 % of the warp slots at 80 registers; an 8-byte load of 32 pixels at an unaligned
-// offset takes up to 3 wavefronts; at 512^2 54, 47 and 45 %: load latency; both before max(-z, 0) u
-// was summed by itself).  Tried and slower: float4
-// records (512^2 59.8 us when planes took 57.7), the rows staged in shared memory by cp.async (86:
-// the copies cost as much as the loads), 32 warps a SM at 64 registers, an L1 prefetch 12 to 32 rows
-// ahead (no change).
+// u and x u, which left rounding in untouched bins: 54.8 and 1537).  At 2048^2 the L1 pipe is at 67 %
+// of its peak, FMA at 62 %, issue 55 %, with 37 % of the warp slots at 80 registers; at 512^2 53, 48 and
+// 46 %: load latency.  An 8-byte load of 32 pixels at an unaligned offset takes up to 3 wavefronts.
+// Tried and slower: float4 records (512^2 59.8 us when planes took 57.7), the rows staged in shared
+// memory by cp.async (86: the copies cost as much as the loads), 32 warps a SM at 64 registers, an L1
+// prefetch 12 to 32 rows ahead (no change).
 // ---------------------------------------------------------------------------
 constexpr int OFW_JOBS = 2, OFW_SEGS = 2, OFW_THREADS = 32 * OFW_JOBS * OFW_SEGS;   // of the batched stage
 
@@ -645,7 +645,8 @@ __device__ __forceinline__ void ofw_body(const OfwArgs &a, const ForwardEpi<floa
             const int it = tj + (e >> 1) * NT, k = kb + it % LN, v = half + 2 * (it / LN) + (e & 1);
             const float *pix = a.ubar + 2 * ((size_t)(v >> 1) * pitch * a.n + ORBIT_PAD) + (v & 1);
             const OrbitJob &job = a.jobs[jb];
-            epi.g[(size_t)job.l[v] * a.M + k] = epi.scale * bin_alone<float>(pix, pitch, a.n, job.am.A, job.am.B, job.am.Op, 32, k);
+            epi.g[(size_t)job.l[v] * a.M + k] =
+                epi.scale * bin_alone<float>(pix, pitch, a.n, job.am.A, job.am.B, job.am.Op, 32, k);
         }
     }
 }
@@ -679,7 +680,8 @@ void launch_forward_orbit_shape(const ctr_plan *p, const float *ub, const Forwar
     auto kern = p->pair_jobs
                     ? (epi.mode == 0 ? k_forward_orbit<2, JOBS, SEGS, true> : k_forward_orbit<2, JOBS, SEGS, false>)
                     : (epi.mode == 0 ? k_forward_orbit<4, JOBS, SEGS, true> : k_forward_orbit<4, JOBS, SEGS, false>);
-    launch_pdl(p->pdl != 0, kern, grid, dim3(32 * JOBS * SEGS), 0, s, OfwArgs{ub, p->d_jobs, p->n, p->M, p->n_jobs, p->job_list[1]}, epi);
+    launch_pdl(p->pdl != 0, kern, grid, dim3(32 * JOBS * SEGS), 0, s,
+               OfwArgs{ub, p->d_jobs, p->n, p->M, p->n_jobs, p->job_list[1]}, epi);
 }
 
 // The launch shape (jobs * 16 + segments): the one ctr_plan_set_fwd_shape set, else the one
