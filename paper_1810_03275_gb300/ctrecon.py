@@ -340,7 +340,8 @@ class Plan:
 
     @property
     def fft_form(self) -> int:
-        """Kernels of the preconditioner passes: 0 warp-level (FP32, n = 256/512/1024), 1 CTA-level."""
+        """Kernels of the preconditioner passes: 0 warp-level (FP32 and BF16, n = 256/512/1024
+        and 16 other sizes from 64 to 864), 1 CTA-level."""
         return int(load().ctr_plan_get_fft_form(self._h))
 
     def set_fft_form(self, form: int):
